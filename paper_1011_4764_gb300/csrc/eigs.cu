@@ -1144,7 +1144,11 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
     w->rot_bytes += P * 3.0 * E.n * es;   // Y and H Y in, X out
     w->rot_flops += 2.0 * 2.0 * P * E.n * E.n;
   }
-  // Gram plan: self pairs over the interior box, chunks of ~1024 points
+  // Gram plan: self pairs over the interior box, chunks of about 1024 points,
+  // fewer (down to 256) where the fragments would leave SMs idle
+  long long gpts = 0;
+  for (const DevFrag& E : w->efr) gpts += (long long)E.ext[0] * E.ext[1] * E.ext[2];
+  const long long gchunk = std::min<long long>(1024, std::max<long long>(256, gpts / (4 * 152)));
   std::vector<HostPair> sp(nf);
   for (int a = 0; a < nf; ++a) {
     const DevFrag& E = w->efr[a];
@@ -1158,7 +1162,7 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
     }
     sp[a].pieces.push_back(pc);
   }
-  make_items_simt(w->efr, sp, 64, 1024, w->gpairs, w->gpieces, w->gitems, w->gpart);
+  make_items_simt(w->efr, sp, 64, gchunk, w->gpairs, w->gpieces, w->gitems, w->gpart);
   w->gblk = 0;
   for (auto& p : w->gpairs) w->gblk = std::max<long long>(w->gblk, p.blk_off + 2LL * w->efr[p.a].n * w->efr[p.b].n);
   // FP32 storage: the same Gram on tensor cores with TF32 hi+lo operands
@@ -1248,10 +1252,10 @@ static ofm_status eig_rr(ofm_ctx* c, int y, int hy, int xo, unsigned long long s
   launch_contract_simt(fp64 ? OFM_PREC_FP64 : OFM_PREC_FP32, fp64, (const DevFrag*)w->d_efr.p,
                        (const DevPair*)w->d_gpairs.p, (const Piece*)w->d_gpieces.p,
                        (const WorkItem*)w->d_gitems.p, (int)w->gitems.size(), w->buf[y].p,
-                       w->buf[hy].p, w->partials.p, 64, s);
+                       w->buf[hy].p, w->partials.p, 64, true, s);
   launch_finalize_simt(fp64 ? OFM_PREC_FP64 : OFM_PREC_FP32, (const DevFrag*)w->d_efr.p,
                        (const DevPair*)w->d_gpairs.p, nf, (const WorkItem*)w->d_gitems.p,
-                       w->partials.p, 64, (double*)w->blocks.p, s);
+                       w->partials.p, 64, (double*)w->blocks.p, true, s);
   }
   const long long mm = (long long)w->mmax * w->mmax;
   { KTimer kt(c, KC_RR);
