@@ -409,7 +409,7 @@ static ofm_status layout_fragments(ofm_ctx* c) {
   OFM_CUDA(c, cudaMemcpyAsync(c->d_frags.p, c->frags.data(), sizeof(DevFrag) * n_frag,
                               cudaMemcpyHostToDevice, c->stream));
   // H-apply launch: 2-D grid (chunks of the largest fragment x fragments)
-  c->agrid = apply_grid(c->frags, es == 8, false, c->stencil_form);
+  c->agrid = apply_grid(c->frags, es == 8, c->stencil_form);
   c->asm_chunk = c->tuned_chunk;
   OFM_TRY(plan_contraction(c));
   // host copies of tables are read back by later calls: wait for the uploads
@@ -911,7 +911,7 @@ extern "C" ofm_status ofm_autotune_assembly(ofm_ctx* c, ofm_precision prec, cons
   o.schedule = 1;
   const bool tcp = prec >= OFM_PREC_TF32;
   for (int form = 1; form <= 2 && st == OFM_OK; ++form) {
-    const ApplyGrid g = apply_grid(c->frags, es == 8, false, form);
+    const ApplyGrid g = apply_grid(c->frags, es == 8, form);
     const bool fits = form == 1 || g.staged;
     for (int i = 0; i < nc && st == OFM_OK; ++i) {
       if (times_ms) times_ms[(form - 1) * nc + i] = -1.0;
@@ -980,7 +980,7 @@ extern "C" ofm_status ofm_autotune_assembly(ofm_ctx* c, ofm_precision prec, cons
   c->stencil_form = st == OFM_OK ? best_form : 0;
   c->tuned_chunk = st == OFM_OK ? best_chunk : 0;
   c->schedule = st == OFM_OK && tcp ? best_sched : 0;
-  c->agrid = apply_grid(c->frags, es == 8, false, c->stencil_form);
+  c->agrid = apply_grid(c->frags, es == 8, c->stencil_form);
   c->asm_chunk = -1;   // re-plan at the next assembly
   if (st != OFM_OK) return st;
   OFM_TRY(ofm_assemble_HS(c, prec, nullptr));

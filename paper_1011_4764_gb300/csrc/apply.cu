@@ -54,24 +54,19 @@ __device__ __forceinline__ int nb_index(int p, int c, int ext, int full, int dir
   return p + (c2 - c) * stride;
 }
 
-// z-marching form of both stencils: a thread owns one (x, y, 16-byte column)
+// z-marching form: a thread owns one (x, y, 16-byte column)
 // of a fragment and walks along z, keeping the planes z-1, z, z+1 of its
 // column in registers; only the plane ahead, the four in-plane neighbours
 // (cache hits: the neighbouring threads load them as their own centre),
-// V and (filter) the previous block are loaded per output.
-// FILTER: fragment mode (interior points only, Chebyshev step);
-// otherwise the a1 apply on every point of the dilated box.
-template <typename T, bool FILTER>
+// and V are loaded per output.
+template <typename T>
 __global__ void __launch_bounds__(256) apply_zmarch_kernel(
     const DevFrag* __restrict__ fr, const T* __restrict__ V, const T* __restrict__ in,
-    const T* __restrict__ prev, T* __restrict__ out, const double* __restrict__ coef, int gx,
-    int gy, int gz, T c0, T c1, int zc) {
+    T* __restrict__ out, int gx, int gy, int gz, T c0, T c1, int zc) {
   using V16 = typename Vec16<T>::type;
   constexpr int VN = Vec16<T>::n;
   __shared__ DevFrag Fs;
-  __shared__ T cf[3];
   if (threadIdx.x == 0) Fs = fr[blockIdx.y];
-  if (FILTER && threadIdx.x < 3) cf[threadIdx.x] = (T)coef[3 * blockIdx.y + threadIdx.x];
   __syncthreads();
   const DevFrag& F = Fs;
   const int qpp = F.ld / VN;
@@ -80,8 +75,6 @@ __global__ void __launch_bounds__(256) apply_zmarch_kernel(
   if (e >= ex * ey * qpp) return;
   const int pxy = e / qpp, q = e - pxy * qpp;
   const int x = pxy % ex, y = pxy / ex;
-  if (FILTER && (x < F.lo[0] || x >= F.lo[0] + F.ext[0] || y < F.lo[1] || y >= F.lo[1] + F.ext[1]))
-    return;
   const int plane = ex * ey;
   // in-plane neighbours (branch-free: outside the storage box -> self, weight 0)
   int nb[4];
@@ -96,13 +89,10 @@ __global__ void __launch_bounds__(256) apply_zmarch_kernel(
     if (nb[i] < 0) nb[i] = pxy;
   }
   const V16* S = reinterpret_cast<const V16*>(in + F.off);
-  const V16* Pv = (FILTER && prev) ? reinterpret_cast<const V16*>(prev + F.off) : nullptr;
   V16* O = reinterpret_cast<V16*>(out + F.off);
-  const T alpha = FILTER ? cf[0] : T(1), beta = FILTER ? cf[1] : T(0), shift = FILTER ? cf[2] : T(0);
-  // this CTA's chunk of planes (blockIdx.z): zc planes of the marched range
-  const int zb = FILTER ? F.lo[2] : 0, ze = FILTER ? F.lo[2] + F.ext[2] : ez;
-  const int z0 = zb + (int)blockIdx.z * zc;
-  const int z1 = min(ze, z0 + zc);
+  // this CTA's chunk of planes (blockIdx.z): zc planes
+  const int z0 = (int)blockIdx.z * zc;
+  const int z1 = min(ez, z0 + zc);
   if (z0 >= z1) return;
   const int X = (F.doff[0] + x) % gx, Y = (F.doff[1] + y) % gy;
   const T* Vrow = V + (long long)Y * gx + X;
@@ -125,12 +115,8 @@ __global__ void __launch_bounds__(256) apply_zmarch_kernel(
 #pragma unroll
     for (int i = 0; i < 4; ++i) sum = fma4(w[i], S[(base + nb[i]) * qpp + q], sum);
     const T v = Vrow[(long long)((F.doff[2] + z) % gz) * vstride];
-    V16 hy = fma4(c0 + v - shift, ctr, zero4(T()));
-    hy = fma4(-c1, sum, hy);
-    V16 o = fma4(alpha, hy, zero4(T()));
-    const int idx = (base + pxy) * qpp + q;
-    if (Pv != nullptr) o = fma4(beta, Pv[idx], o);
-    O[idx] = o;
+    V16 hy = fma4(c0 + v, ctr, zero4(T()));
+    O[(base + pxy) * qpp + q] = fma4(-c1, sum, hy);
     below = ctr;
     ctr = above;
   }
@@ -143,36 +129,31 @@ __global__ void __launch_bounds__(256) apply_zmarch_kernel(
 // dimension wraps) into a ring of STG_BUF plane buffers, completing on the
 // buffer's mbarrier; a slot is refilled as soon as its plane is no longer
 // needed, so up to three planes per CTA are in flight while it computes.  All six neighbours then
-// come from shared memory; V and (filter) the previous block stream from
-// global memory into registers one plane ahead of their use.  Staged rows outside a non-periodic storage box are zeroed
+// come from shared memory; V streams from global memory into registers one
+// plane ahead of its use.  Staged rows outside a non-periodic storage box are zeroed
 // once; planes outside it complete their barrier phase without a copy and
 // are skipped in the sum.
 constexpr int STG_BUF = 5;
 constexpr int STG_THREADS = 256;
 constexpr int STG_EPT = 4;   // tile elements per thread (16 bytes each)
 
-template <typename T, bool FILTER>
+template <typename T>
 __global__ void __launch_bounds__(STG_THREADS) apply_staged_kernel(
     const DevFrag* __restrict__ fr, const T* __restrict__ V, const T* __restrict__ in,
-    const T* __restrict__ prev, T* __restrict__ out, const double* __restrict__ coef, int gx,
-    int gy, int gz, T c0, T c1, int ty, int zc, int* flag) {
+    T* __restrict__ out, int gx, int gy, int gz, T c0, T c1, int ty, int zc, int* flag) {
   using namespace ptx;
   using V16 = typename Vec16<T>::type;
   constexpr int VN = Vec16<T>::n;
   extern __shared__ __align__(128) unsigned char stg_smem[];
   __shared__ DevFrag Fs;
-  __shared__ T cf[3];
   __shared__ __align__(8) unsigned long long mbar[STG_BUF];
   const int tid = threadIdx.x;
   if (tid == 0) Fs = fr[blockIdx.y];
-  if (FILTER && tid < 3) cf[tid] = (T)coef[3 * blockIdx.y + tid];
   __syncthreads();
   const DevFrag& F = Fs;
   const int ex = F.dext[0], ey = F.dext[1], ez = F.dext[2];
-  const int yb = FILTER ? F.lo[1] : 0, ye = FILTER ? F.lo[1] + F.ext[1] : ey;
-  const int zb = FILTER ? F.lo[2] : 0, ze = FILTER ? F.lo[2] + F.ext[2] : ez;
-  const int y0 = yb + (int)blockIdx.x * ty, y1 = min(ye, y0 + ty);
-  const int z0 = zb + (int)blockIdx.z * zc, z1 = min(ze, z0 + zc);
+  const int y0 = (int)blockIdx.x * ty, y1 = min(ey, y0 + ty);
+  const int z0 = (int)blockIdx.z * zc, z1 = min(ez, z0 + zc);
   if (y0 >= y1 || z0 >= z1) return;   // uniform over the CTA
   const int qpp = F.ld / VN;
   const int rows = y1 - y0 + 2;                 // staged rows y0-1 .. y1
@@ -240,11 +221,8 @@ __global__ void __launch_bounds__(STG_THREADS) apply_staged_kernel(
     for (int p = z0 - 1; p < pnext; ++p) issue(p);
   int pwait = z0 - 1;     // planes < pwait have been waited for
 
-  const int nx = FILTER ? F.ext[0] : ex, xo = FILTER ? F.lo[0] : 0;
-  const int per_row = nx * qpp;
+  const int per_row = ex * qpp;
   const int nel = (y1 - y0) * per_row;   // <= STG_THREADS * STG_EPT (host's tile choice)
-  const T alpha = FILTER ? cf[0] : T(1), beta = FILTER ? cf[1] : T(0), shift = FILTER ? cf[2] : T(0);
-  const V16* Pv = (FILTER && prev) ? reinterpret_cast<const V16*>(prev + F.off) : nullptr;
   V16* O = reinterpret_cast<V16*>(out + F.off);
   const long long vplane = (long long)gx * gy;
   const int rowq = ex * qpp;   // 16-byte elements of one staged row
@@ -256,38 +234,29 @@ __global__ void __launch_bounds__(STG_THREADS) apply_staged_kernel(
     const int ee = e < nel ? e : 0;
     const int yl = ee / per_row;
     const int rem = ee - yl * per_row;
-    const int xl = rem / qpp, q = rem - xl * qpp;
-    const int x = xo + xl, y = y0 + yl;
+    const int x = rem / qpp, q = rem - x * qpp;
+    const int y = y0 + yl;
     xs[u] = x;
     sidx[u] = (yl + 1) * rowq + x * qpp + q;
     gidx[u] = (y * ex + x) * qpp + q;
     vidx[u] = ((F.doff[1] + y) % gy) * gx + (F.doff[0] + x) % gx;
   }
   const long long gplane = (long long)ey * ex * qpp;   // 16-byte elements of one storage plane
-  // the previous block and V of the plane being computed, loaded one iteration ahead
-  V16 pv[STG_EPT];
+  // V of the plane being computed, loaded one iteration ahead
   T vv[STG_EPT];
   auto prefetch = [&](int z) {
-    const long long zo = (long long)z * gplane;
     const long long zv = (long long)((F.doff[2] + z) % gz) * vplane;
 #pragma unroll
     for (int u = 0; u < STG_EPT; ++u) {
-      if (tid + u * STG_THREADS < nel) {
-        vv[u] = V[zv + vidx[u]];
-        if (Pv != nullptr) pv[u] = Pv[zo + gidx[u]];
-      }
+      if (tid + u * STG_THREADS < nel) vv[u] = V[zv + vidx[u]];
     }
   };
   prefetch(z0);
   bool ok = true;
   for (int z = z0; z < z1; ++z) {
-    V16 pvc[STG_EPT];
     T vc[STG_EPT];
 #pragma unroll
-    for (int u = 0; u < STG_EPT; ++u) {
-      pvc[u] = pv[u];
-      vc[u] = vv[u];
-    }
+    for (int u = 0; u < STG_EPT; ++u) vc[u] = vv[u];
     if (z + 1 < z1) prefetch(z + 1);
     // planes z-1, z, z+1 must have landed
     while (ok && pwait <= z + 1) {
@@ -314,15 +283,8 @@ __global__ void __launch_bounds__(STG_THREADS) apply_staged_kernel(
       if (xm >= 0) sum = add4(sum, Bc[sc + (xm - x) * qpp]);
       if (has_b) sum = add4(sum, Bb[sc]);
       if (has_a) sum = add4(sum, Ba[sc]);
-      V16 hy = fma4(c0 + vc[u] - shift, Bc[sc], zero4(T()));
-      hy = fma4(-c1, sum, hy);
-      if constexpr (FILTER) {
-        V16 o = fma4(alpha, hy, zero4(T()));
-        if (Pv != nullptr) o = fma4(beta, pvc[u], o);
-        O[zo + gidx[u]] = o;
-      } else {
-        O[zo + gidx[u]] = hy;
-      }
+      V16 hy = fma4(c0 + vc[u], Bc[sc], zero4(T()));
+      O[zo + gidx[u]] = fma4(-c1, sum, hy);
     }
     __syncthreads();   // slot of plane z-1 is free
     if (tid == 0 && pnext <= plast) issue(pnext);
@@ -341,7 +303,7 @@ __global__ void __launch_bounds__(STG_THREADS) apply_staged_kernel(
 // SM, else one) and at most STG_EPT elements per thread, and the chunk count
 // fills about two resident waves of the GB300 (152 SMs).  Register form (fallback when even one row does not fit):
 // x covers the (x, y, column group) elements of the largest plane.
-ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, bool filter, int form) {
+ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, int form) {
   const int vn = fp64 ? 2 : 4;
   const int es = fp64 ? 8 : 4;
   const int sms = 152;
@@ -350,11 +312,11 @@ ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, bool filter, int
   for (const DevFrag& f : fr) {
     const long long xy = (long long)f.dext[0] * f.dext[1] * (f.ld / vn);
     mx = std::max(mx, xy);
-    threads += filter ? (long long)f.ext[0] * f.ext[1] * (f.ld / vn) : xy;
-    zmax = std::max(zmax, filter ? f.ext[2] : f.dext[2]);
-    ymax = std::max(ymax, filter ? f.ext[1] : f.dext[1]);
+    threads += xy;
+    zmax = std::max(zmax, f.dext[2]);
+    ymax = std::max(ymax, f.dext[1]);
     rowB = std::max(rowB, (long long)f.dext[0] * f.ld * es);
-    rowQ = std::max(rowQ, (long long)(filter ? f.ext[0] : f.dext[0]) * (f.ld / vn));
+    rowQ = std::max(rowQ, (long long)f.dext[0] * (f.ld / vn));
   }
   ApplyGrid g;
   // staged form where the caller (form 2), or with form 0 OFM_STENCIL=staged,
@@ -381,7 +343,7 @@ ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, bool filter, int
       g.smem = (int)((long long)STG_BUF * (best + 2) * rowB);
       const int per_sm = bi == 0 ? 2 : 1;
       long long per_chunk = 0;
-      for (const DevFrag& f : fr) per_chunk += ((filter ? f.ext[1] : f.dext[1]) + best - 1) / best;
+      for (const DevFrag& f : fr) per_chunk += (f.dext[1] + best - 1) / best;
       const long long nch = std::max(1LL, std::min<long long>(zmax, (2LL * sms * per_sm + per_chunk - 1) / per_chunk));
       g.zc = (int)((zmax + nch - 1) / nch);
       g.z = (zmax + g.zc - 1) / g.zc;
@@ -390,10 +352,7 @@ ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, bool filter, int
   }
   if (g.staged) {
     // once per plan (the call is not free: kept out of the launch path)
-    const void* k = fp64 ? (filter ? (const void*)apply_staged_kernel<double, true>
-                                   : (const void*)apply_staged_kernel<double, false>)
-                         : (filter ? (const void*)apply_staged_kernel<float, true>
-                                   : (const void*)apply_staged_kernel<float, false>);
+    const void* k = fp64 ? (const void*)apply_staged_kernel<double> : (const void*)apply_staged_kernel<float>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem) == cudaSuccess)
       return g;
     cudaGetLastError();   // not available: the register form below
@@ -408,230 +367,24 @@ ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, bool filter, int
   return g;
 }
 
-template <typename T, bool FILTER>
+template <typename T>
 static void zmarch(const ApplyGrid& ag, int nfrag, const DevFrag* d_fr, const void* V,
-                   const void* in, const void* prev, void* out, const double* coef,
-                   const int gn[3], double h, int* flag, cudaStream_t s) {
+                   const void* in, void* out, const int gn[3], double h, int* flag, cudaStream_t s) {
   const double c0 = 3.0 / (h * h), c1 = 0.5 / (h * h);
   dim3 g(ag.x, nfrag, ag.z);
-  if (ag.staged) {
-    apply_staged_kernel<T, FILTER><<<g, STG_THREADS, ag.smem, s>>>(
-        d_fr, (const T*)V, (const T*)in, (const T*)prev, (T*)out, coef, gn[0], gn[1], gn[2],
-        (T)c0, (T)c1, ag.ty, ag.zc, flag);
-  } else {
-    apply_zmarch_kernel<T, FILTER><<<g, 256, 0, s>>>(d_fr, (const T*)V, (const T*)in,
-                                                     (const T*)prev, (T*)out, coef, gn[0], gn[1],
-                                                     gn[2], (T)c0, (T)c1, ag.zc);
-  }
+  if (ag.staged)
+    apply_staged_kernel<T><<<g, STG_THREADS, ag.smem, s>>>(d_fr, (const T*)V, (const T*)in, (T*)out, gn[0], gn[1],
+                                                          gn[2], (T)c0, (T)c1, ag.ty, ag.zc, flag);
+  else
+    apply_zmarch_kernel<T><<<g, 256, 0, s>>>(d_fr, (const T*)V, (const T*)in, (T*)out, gn[0], gn[1], gn[2],
+                                             (T)c0, (T)c1, ag.zc);
 }
 
 void launch_apply_global(const DevFrag* d_fr, int nfrag, const ApplyGrid& g, const void* V,
                          const void* states, void* hphi, const int gn[3], double h, bool fp64,
                          int* flag, cudaStream_t s) {
-  if (fp64) zmarch<double, false>(g, nfrag, d_fr, V, states, nullptr, hphi, nullptr, gn, h, flag, s);
-  else zmarch<float, false>(g, nfrag, d_fr, V, states, nullptr, hphi, nullptr, gn, h, flag, s);
-}
-
-// a0, fragment mode: the fragment Hamiltonian is the principal submatrix of
-// H on the box, so only interior points are written (the zero halo stays
-// zero) and the stencil reads zeros beyond the box.  One fused step of the
-// scaled Chebyshev three-term recurrence:
-//     out = alpha_f * (H_f in - c_f in) + beta_f * prev
-// with per-fragment coefficients coef[f] = (alpha, beta, c); prev may be
-// null when beta is zero.
-void launch_apply_filter(const DevFrag* d_fr, int nfrag, const ApplyGrid& g, const void* V,
-                         const void* in, const void* prev, void* out, const double* coef,
-                         const int gn[3], double h, bool fp64, int* flag, cudaStream_t s) {
-  if (fp64) zmarch<double, true>(g, nfrag, d_fr, V, in, prev, out, coef, gn, h, flag, s);
-  else zmarch<float, true>(g, nfrag, d_fr, V, in, prev, out, coef, gn, h, flag, s);
-}
-
-// ------------------------------------------------ whole filter on chip ----
-//
-// The whole degree-d Chebyshev filter of one fragment and ONE state column
-// in one CTA (FP32 storage, interior box EX x EY x EZ fixed at compile
-// time): the column's box is loaded once, every step runs between registers
-// and shared memory, and the filtered column Y = p(H_f) X and H_f Y leave
-// once.  The stencil acts on each state column independently, so the CTAs
-// of a fragment's columns share nothing.  Against one launch per degree
-// (three blocks through HBM per step) the HBM traffic of a filter drops from
-// ~3 d blocks to ~3 blocks; a step is bound by shared memory (four in-plane
-// neighbour loads and one store per point) and instruction issue.
-//   - two threads own each interior column (x, y), the lower and the upper
-//     half of its z range, and keep their half of the current iterate in
-//     registers; z neighbours come from registers (the two middle and the
-//     wrap-around ones from shared memory), in-plane neighbours from the
-//     shared copy of the current iterate;
-//   - the shared copy is the interior box ([z][y][x], unpadded: the two rows
-//     of 16 points a warp covers are 32 consecutive words, conflict-free) in
-//     two buffers: a step reads one and writes the next iterate over the
-//     previous one in the other (each point is read and rewritten by its own
-//     thread), one barrier per step.  c0 + V of every point sits in a third
-//     area;
-//   - a missing in-plane neighbour (non-periodic edge) reads the point itself
-//     with weight 0 and a periodic one reads the wrapped point, exactly as in
-//     apply_zmarch_kernel's filter mode, whose arithmetic and order are kept:
-//     both forms give the same values.
-template <int EX, int EY, int EZ>
-struct CfBox {
-  static constexpr int NXY = EX * EY;                 // points per plane (unpadded)
-  static constexpr int ZH = EZ / 2, NT = 2 * NXY;     // two threads per z-column
-  // two copies of the iterate, then c0 + V of every interior point
-  static constexpr size_t smem = 3 * (size_t)EZ * NXY * sizeof(float);
-};
-
-// One step for the ZH planes of a thread.  src holds the current iterate
-// (also in cur), dst the previous one; the next iterate replaces the
-// previous one in dst point by point (only this thread reads those points
-// of dst during the step) and replaces cur.  nb[i], w[i]: in-plane
-// neighbour offsets and 0/1 weights (x+1, x-1, y+1, y-1; a missing
-// neighbour reads the point itself with weight 0, as in the HBM form); ob /
-// oa: offsets of the planes just below / above the thread's range (-1:
-// zero there).  With write = false (the final H Y) the result goes to cur
-// only and dst is untouched.
-template <int EX, int EY, int EZ>
-__device__ __forceinline__ void cf_step(const float* __restrict__ src, float* __restrict__ dst,
-                                        int own, int ob, int oa, const int (&nb)[4],
-                                        const float (&w)[4], float (&cur)[CfBox<EX, EY, EZ>::ZH],
-                                        const float* __restrict__ vc, float c1, float al, float be,
-                                        float sh, bool has_prev, bool write) {
-  using B = CfBox<EX, EY, EZ>;
-  float below = ob >= 0 ? src[ob] : 0.f;
-  const float edge_a = oa >= 0 ? src[oa] : 0.f;
-  const float* p0 = src + nb[0];
-  const float* p1 = src + nb[1];
-  const float* p2 = src + nb[2];
-  const float* p3 = src + nb[3];
-  float* d = dst + own;
-#pragma unroll
-  for (int z = 0; z < B::ZH; ++z) {
-    const float above = (z + 1 < B::ZH) ? cur[z + 1] : edge_a;
-    float sum = below + above;
-    sum = fmaf(w[0], p0[z * B::NXY], sum);
-    sum = fmaf(w[1], p1[z * B::NXY], sum);
-    sum = fmaf(w[2], p2[z * B::NXY], sum);
-    sum = fmaf(w[3], p3[z * B::NXY], sum);
-    float h = fmaf(vc[z * B::NXY] - sh, cur[z], 0.f);
-    h = fmaf(-c1, sum, h);
-    float o = fmaf(al, h, 0.f);
-    if (has_prev) o = fmaf(be, d[z * B::NXY], o);
-    below = cur[z];   // the old value is the next point's lower neighbour
-    cur[z] = o;
-    if (write) d[z * B::NXY] = o;
-  }
-}
-
-template <int EX, int EY, int EZ>
-__global__ void __launch_bounds__(2 * EX * EY, 1) cheb_filter_kernel(
-    const DevFrag* __restrict__ fr, const float* __restrict__ V, const float* __restrict__ X,
-    float* __restrict__ Y, float* __restrict__ HY, const double* __restrict__ coef, int nsteps,
-    int nfrag, int gx, int gy, int gz, float c0, float c1) {
-  using B = CfBox<EX, EY, EZ>;
-  constexpr int ZH = B::ZH;
-  extern __shared__ float cf_box[];
-  const int f = blockIdx.y, j = blockIdx.x;
-  const DevFrag F = fr[f];
-  if (j >= F.n) return;   // uniform over the CTA
-  const int t = threadIdx.x;
-  const int c = t % B::NXY, half = t / B::NXY;
-  const int x = c % EX, y = c / EX, z0 = half * ZH;
-  const bool fz = F.full[2] != 0;
-  const int own = z0 * B::NXY + c;
-  const int ob = z0 > 0 ? own - B::NXY : (fz ? (EZ - 1) * B::NXY + c : -1);
-  const int oa = z0 + ZH < EZ ? own + ZH * B::NXY : (fz ? c : -1);
-  // in-plane neighbours within the interior plane (full dimensions wrap)
-  int nb[4];
-  float w[4];
-  {
-    const int xp = x + 1 < EX ? c + 1 : (F.full[0] ? c + 1 - EX : -1);
-    const int xm = x > 0 ? c - 1 : (F.full[0] ? c - 1 + EX : -1);
-    const int yp = y + 1 < EY ? c + EX : (F.full[1] ? c + EX - B::NXY : -1);
-    const int ym = y > 0 ? c - EX : (F.full[1] ? c - EX + B::NXY : -1);
-    const int q[4] = {xp, xm, yp, ym};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      w[i] = q[i] >= 0 ? 1.f : 0.f;
-      nb[i] = (q[i] >= 0 ? q[i] : c) + z0 * B::NXY;
-    }
-  }
-  const long long pstride = (long long)F.dext[0] * F.dext[1];   // storage points per plane
-  const long long p0 =
-      ((long long)(F.lo[2] + z0) * F.dext[1] + (F.lo[1] + y)) * F.dext[0] + F.lo[0] + x;
-  float* vcs = cf_box + 2 * EZ * B::NXY + own;   // c0 + V, plane stride NXY
-  {
-    const float* Vrow = V + (long long)((F.doff[1] + F.lo[1] + y) % gy) * gx + (F.doff[0] + F.lo[0] + x) % gx;
-    const long long vstride = (long long)gx * gy;
-#pragma unroll
-    for (int z = 0; z < ZH; ++z)
-      vcs[z * B::NXY] = c0 + Vrow[(long long)((F.doff[2] + F.lo[2] + z0 + z) % gz) * vstride];
-  }
-  float cur[ZH];
-#pragma unroll
-  for (int z = 0; z < ZH; ++z) cur[z] = X[F.off + (p0 + z * pstride) * F.ld + j];
-#pragma unroll
-  for (int z = 0; z < ZH; ++z) cf_box[own + z * B::NXY] = cur[z];
-  __syncthreads();
-  float* b0 = cf_box;
-  float* b1 = cf_box + EZ * B::NXY;
-  const double* cf = coef + 3 * (size_t)f;
-  float* src = b0;
-  float* dst = b1;
-  for (int k = 0; k < nsteps; ++k) {
-    const double* ca = cf + 3 * (size_t)k * nfrag;
-    cf_step<EX, EY, EZ>(src, dst, own, ob, oa, nb, w, cur, vcs, c1, (float)ca[0], (float)ca[1],
-                        (float)ca[2], k > 0, true);
-    __syncthreads();
-    float* tmp = src;
-    src = dst;
-    dst = tmp;
-  }
-  // cur holds the filtered column Y (also in src); H_f Y (alpha 1, beta 0,
-  // shift 0) goes to the registers of a second pass, Y straight out first
-  if (Y) {
-#pragma unroll
-    for (int z = 0; z < ZH; ++z) Y[F.off + (p0 + z * pstride) * F.ld + j] = cur[z];
-  }
-  cf_step<EX, EY, EZ>(src, dst, own, ob, oa, nb, w, cur, vcs, c1, 1.f, 0.f, 0.f, false, false);
-#pragma unroll
-  for (int z = 0; z < ZH; ++z) HY[F.off + (p0 + z * pstride) * F.ld + j] = cur[z];
-}
-
-// Box shapes with an on-chip filter: every fragment must have this interior
-// shape, and a full dimension must coincide with the storage box.
-static bool cf_shape(const std::vector<DevFrag>& frags, int ex, int ey, int ez) {
-  for (const DevFrag& F : frags) {
-    if (F.ext[0] != ex || F.ext[1] != ey || F.ext[2] != ez) return false;
-    for (int d = 0; d < 3; ++d)
-      if (F.full[d] && (F.ext[d] != F.dext[d] || F.lo[d] != 0)) return false;
-  }
-  return !frags.empty();
-}
-
-// Dynamic shared memory of the on-chip filter for these fragments, or 0 when
-// it does not apply (FP64 storage, or a box shape without a compiled form).
-size_t cheb_filter_smem(const std::vector<DevFrag>& frags, bool fp64) {
-  if (fp64) return 0;
-  if (cf_shape(frags, 16, 32, 32)) return CfBox<16, 32, 32>::smem;
-  return 0;
-}
-
-// One launch per filter: CTA (state j, fragment f) for every j < m_f.  Y may
-// be null (only H X wanted: nsteps = 0).
-void launch_cheb_filter(const DevFrag* d_fr, int nfrag, int mmax, size_t smem, const void* V,
-                        const void* X, void* Y, void* HY, const double* coef, int nsteps,
-                        const int gn[3], double h, cudaStream_t s) {
-  const double c0 = 3.0 / (h * h), c1 = 0.5 / (h * h);
-  if (smem == CfBox<16, 32, 32>::smem) {
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(cheb_filter_kernel<16, 32, 32>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attr = true;
-    }
-    cheb_filter_kernel<16, 32, 32><<<dim3(mmax, nfrag), CfBox<16, 32, 32>::NT, smem, s>>>(
-        d_fr, (const float*)V, (const float*)X, (float*)Y, (float*)HY, coef, nsteps, nfrag,
-        gn[0], gn[1], gn[2], (float)c0, (float)c1);
-  }
+  if (fp64) zmarch<double>(g, nfrag, d_fr, V, states, hphi, gn, h, flag, s);
+  else zmarch<float>(g, nfrag, d_fr, V, states, hphi, gn, h, flag, s);
 }
 
 // ------------------------------------------------------------ conversions --

@@ -109,7 +109,7 @@ struct ApplyGrid {
 };
 // form: 0 register form unless OFM_STENCIL=staged, 1 register form, 2 staged
 // form where it fits (else the register form)
-ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, bool filter, int form = 0);
+ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, int form = 0);
 // flag: set to 1 when a bounded wait of the staged form gives up
 void launch_apply_global(const DevFrag* d_fr, int nfrag, const ApplyGrid& g, const void* V,
                          const void* states, void* hphi, const int gn[3], double h, bool fp64,
@@ -118,15 +118,8 @@ void launch_import_states(const DevFrag* d_fr, int a, const DevFrag& fa, const d
                           void* states, bool fp64, cudaStream_t s);
 void launch_export_states(const DevFrag& fa, const void* states, double* dst, bool fp64,
                           bool dilated_hphi, cudaStream_t s);
-size_t cheb_filter_smem(const std::vector<DevFrag>& frags, bool fp64);
 void launch_select_states(const DevFrag& Fo, const DevFrag& Fn, int first, const void* src,
                           void* dst, bool fp64, cudaStream_t s);
-void launch_cheb_filter(const DevFrag* d_fr, int nfrag, int mmax, size_t smem, const void* V,
-                        const void* X, void* Y, void* HY, const double* coef, int nsteps,
-                        const int gn[3], double h, cudaStream_t s);
-void launch_apply_filter(const DevFrag* d_fr, int nfrag, const ApplyGrid& g, const void* V,
-                         const void* in, const void* prev, void* out, const double* coef,
-                         const int gn[3], double h, bool fp64, int* flag, cudaStream_t s);
 void launch_convert_V(const double* src, void* dst, long long n, bool fp64, cudaStream_t s);
 void launch_contract_simt(int prec, bool store_fp64, const DevFrag* d_fr, const DevPair* d_pairs,
                           const Piece* d_pieces, const WorkItem* d_items, int nitems,
@@ -137,6 +130,57 @@ void launch_finalize_simt(int prec, const DevFrag* d_fr, const DevPair* d_pairs,
                           double* blocks, bool upper, cudaStream_t s);
 void launch_scatter_dense(const DevFrag* d_fr, const DevPair* d_pairs, int npairs,
                           const double* blocks, int n, double* Hd, double* Sd, cudaStream_t s);
+
+// A fragment's block in the eigensolver: state-major vectors of the box's
+// points (eigblk.cu).
+struct EigFrag {
+  int e[3];         // extents along the layout's axes, fastest first
+  int e0p;          // e[0] padded to a multiple of four
+  int full[3];      // 1 where the box spans the grid along that axis
+  int ax[3];        // grid dimension of each layout axis
+  int n;            // vectors
+  int Ps;           // elements from one vector to the next (multiple of 4)
+  long long off;    // first element in the block arenas
+  long long voff;   // first element in the c0 + V arena
+};
+struct EigFilterPlan {
+  int S = 0;              // steps per launch at most; 0: one step per launch over HBM
+  bool even = true;       // every box splits into whole 4 x 2 patches
+  int threads = 0;
+  size_t smem = 0;
+  std::vector<int4> jobs;
+};
+struct EigGramPlan {
+  std::vector<int4> items;
+  std::vector<long long> part_off, blk_off;
+  std::vector<int2> fitems;
+  long long part_elems = 0, blk_elems = 0;
+  int KP = 32;
+  size_t smem = 0;
+};
+void eig_layout(const std::vector<DevFrag>& fr, const std::vector<int>& m,
+                std::vector<EigFrag>& out, long long& elems, long long& vc_elems);
+void eig_filter_plan(const std::vector<EigFrag>& ef, bool fp64, EigFilterPlan& plan);
+void eig_gram_plan(const std::vector<EigFrag>& ef, bool fp64, EigGramPlan& plan);
+void eig_rotate_plan(const std::vector<EigFrag>& ef, bool fp64, int& blocks, size_t& smem);
+void launch_eig_init(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<EigFrag>& ef, void* X,
+                     unsigned long long seed, bool fp64, cudaStream_t s);
+void launch_eig_vc(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<EigFrag>& ef, const void* V,
+                   const int gn[3], double h, void* vc, bool fp64, cudaStream_t s);
+// Filter of degree deg from the block in A (B: workspace, both overwritten),
+// then H Y.  Returns 0 when H Y is in A and Y in B, 1 when the other way round.
+int launch_eig_filter(const EigFilterPlan& plan, const EigFrag* d_ef, const std::vector<EigFrag>& ef,
+                      const int4* d_jobs, void* A, void* B, const void* vc, const double* coef, int deg,
+                      int plain_slot, bool fp64, double h, cudaStream_t s, int* launches);
+void launch_eig_gram(const EigGramPlan& g, const EigFrag* d_ef, int nfrag, const int4* d_items,
+                     const long long* d_part_off, const int2* d_fitems, const long long* d_blk_off,
+                     const void* Y, const void* HY, void* partials, double* blocks, bool fp64, cudaStream_t s);
+void launch_eig_rotate(const EigFrag* d_ef, const DevFrag* d_fr, int nfrag, int blocks, size_t smem,
+                       const void* Y, const void* HY, void* Xo, const double* Cm, long long cstride,
+                       const int* rank, const double* theta, const long long* toff, double* partial,
+                       int mstride, unsigned long long salt, double* res, bool fp64, cudaStream_t s);
+void launch_eig_export(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<EigFrag>& ef, int nmax,
+                       const void* X, void* sgn, int mstride, void* states, bool fp64, cudaStream_t s);
 
 }  // namespace ofm
 
