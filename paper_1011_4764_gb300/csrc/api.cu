@@ -38,6 +38,7 @@ ofm_status ofm_ensure(ofm_ctx* c, DevBuf& b, size_t bytes, const char* what) {
     return ofm_fail(c, OFM_ERR_OOM, buf);
   }
   if (b.p) {
+    if (c) ++c->buf_gen;   // captured assemblies may hold the old address
     cudaError_t e = cudaFree(b.p);
     b.p = nullptr;
     b.cap = 0;
@@ -740,10 +741,9 @@ static ofm_status prepare_assembly(ofm_ctx* c, ofm_precision prec, int sched) {
   if (sched == 2 && !region_schedule(c, prec, sched))
     return ofm_fail(c, OFM_ERR_INVALID, std::string("region schedule unavailable: ") + ofm_region_why(c));
   if (region_schedule(c, prec, sched)) return ofm_region_prepare(c, prec);   // tables and buffers
+  if (prec != OFM_PREC_FP64 && prec != OFM_PREC_FP32) return ofm_tc_prepare(c, prec);
   OFM_TRY(ensure_hphi(c));
-  if (prec == OFM_PREC_FP64 || prec == OFM_PREC_FP32)
-    OFM_TRY(ofm_ensure_big(c, c->partials, sizeof(double) * c->simt_partial_elems, "partials"));
-  return OFM_OK;
+  return ofm_ensure_big(c, c->partials, sizeof(double) * c->simt_partial_elems, "partials");
 }
 
 // The launches of one assembly (a1 apply, a3/a4 contraction, a5 blocks) on
@@ -753,9 +753,9 @@ static ofm_status enqueue_assembly(ofm_ctx* c, ofm_precision prec, int sched) {
     c->last_schedule = 2;
     return ofm_region_run(c, prec);
   }
-  OFM_TRY(ofm_apply_h(c));
   c->last_schedule = 1;
   if (prec == OFM_PREC_FP64 || prec == OFM_PREC_FP32) {
+    OFM_TRY(ofm_apply_h(c));
     { KTimer t(c, KC_CONTRACT, 1, c->contract_bytes, (double)c->flops);
     launch_contract_simt(prec, c->storage == OFM_STORE_FP64, (const DevFrag*)c->d_frags.p,
                          (const DevPair*)c->d_pairs.p, (const Piece*)c->d_pieces.p,
@@ -796,6 +796,7 @@ static ofm_status capture_assembly(ofm_ctx* c, ofm_precision prec, int sched) {
   }
   c->asm_tc[prec] = c->tc_check;
   c->asm_sched[prec] = sched;
+  c->asm_gen[prec] = c->buf_gen;
   c->tc_check = false;
   c->stencil_check = false;
   if (st != OFM_OK || e != cudaSuccess || !g ||
@@ -834,7 +835,7 @@ static ofm_status ofm_assemble_HS_impl(ofm_ctx* c, ofm_precision prec, const ofm
   OFM_TRY(prepare_assembly(c, prec, sched));
   const bool held = c->hold_tc && region_schedule(c, prec, sched) && prec != OFM_PREC_FP64 &&
                     prec != OFM_PREC_FP32;   // one direct launch
-  if (c->asm_exec[prec] && c->asm_sched[prec] != sched) {
+  if (c->asm_exec[prec] && (c->asm_sched[prec] != sched || c->asm_gen[prec] != c->buf_gen)) {
     cudaGraphExecDestroy(c->asm_exec[prec]);
     c->asm_exec[prec] = nullptr;
   }
@@ -847,7 +848,7 @@ static ofm_status ofm_assemble_HS_impl(ofm_ctx* c, ofm_precision prec, const ofm
         c->prof.st[k].bytes += c->asm_cost[prec][k].bytes;
         c->prof.st[k].flops += c->asm_cost[prec][k].flops;
       }
-      c->stencil_check = !region_schedule(c, prec, sched);
+      c->stencil_check = !region_schedule(c, prec, sched) && (prec == OFM_PREC_FP64 || prec == OFM_PREC_FP32);
       if (c->asm_tc[prec]) c->tc_check = true;
       c->last_schedule = region_schedule(c, prec, sched) ? 2 : 1;
       c->assembled = true;

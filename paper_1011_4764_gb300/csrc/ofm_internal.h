@@ -51,6 +51,18 @@ struct Piece {
   int len[3];      // extent
 };
 
+// Operand planes of one fragment over one box of the grid (a coverage region,
+// or the fragment's own storage box for the pair schedule).
+struct RUnit {
+  int frag;
+  int s0[3];          // start (global grid coordinates)
+  int L[3];           // extent
+  int p8;             // plane stride in K: L[0] * L[1] rounded up to 8
+  int ntiles;         // 64-point tiles: (L[2] * p8) / 64 rounded up
+  long long tile0;    // first global tile of this unit
+  long long base;     // byte offset of the block in the plane arena
+};
+
 struct DevPair {
   int a, b;
   int item0, nitem;     // work items of this pair (contiguous)
@@ -286,6 +298,8 @@ struct ofm_ctx {
   ofm::KStat asm_cost[5][ofm::KC_COUNT];
   bool asm_tc[5] = {false, false, false, false, false};
   int asm_sched[5] = {0, 0, 0, 0, 0};   // schedule each graph was captured with
+  unsigned buf_gen = 0;             // device buffers re-allocated so far ...
+  unsigned asm_gen[5] = {0, 0, 0, 0, 0};   // ... when each graph was captured
   bool graphs_off = false;          // capture failed once on this stream: launch directly
   bool tc_check = false;            // a tensor-core launch's timeout flag is unread
   bool stencil_check = false;       // a stencil launch's timeout flag is unread
@@ -355,22 +369,18 @@ ofm_status ofm_ensure_big(ofm_ctx* c, ofm::DevBuf& b, size_t bytes, const char* 
 // cross-translation-unit steps
 ofm_status ofm_apply_h(ofm_ctx* c);
 ofm_status ofm_make_dense(ofm_ctx* c);
-ofm_status ofm_plan_extra(ofm_ctx* c);        // tensor-core plan after a build
+ofm_status ofm_plan_extra(ofm_ctx* c);        // tensor-core pair plan after a build
 void ofm_free_extra(ofm_ctx* c);              // frees eig and tc
 void ofm_eig_free(ofm_ctx* c);
 void ofm_prof_release(ofm_ctx* c);            // waits for and frees timing events
 void ofm_tc_free(ofm_ctx* c);
 ofm_status ofm_contract_tc(ofm_ctx* c, ofm_precision prec);
-// tensor-core plans over any fragment table (assembly, eigensolver Gram)
-enum { OFM_TC_TF32 = 0, OFM_TC_BF16 = 1, OFM_TC_BF16X3 = 2, OFM_TC_TF32X3 = 3 };
-ofm_status ofm_tc_plan_build(ofm_ctx* c, struct TcPlan** tp, const std::vector<ofm::DevFrag>& fr,
-                             const std::vector<ofm::HostPair>& pairs,
-                             const std::vector<long long>& blk_off, long long kh, long long chunk);
-ofm_status ofm_tc_run(ofm_ctx* c, struct TcPlan* t, int kind, const ofm::DevFrag* d_frags,
-                      const void* states, const void* hphi, double* blocks, int kclass_contract,
-                      int kclass_finalize, double bytes, double flops);
-bool ofm_tc_plan_ok(const struct TcPlan* t, int kind);   // the kind's staging fits
+// tensor-core contraction of the pair schedule (tc.cu)
+ofm_status ofm_tc_prepare(ofm_ctx* c, ofm_precision prec);   // device tables and buffers
 void ofm_tc_plan_free(struct TcPlan* t);
+ofm_status ofm_pair_planes(ofm_ctx* c, long long bytes, void** arena);
+ofm_status ofm_pair_pack(ofm_ctx* c, int kind, const ofm::RUnit* units, const int4* cta, int ncta,
+                         void* arena, long long bytes);
 ofm_status ofm_wait_status(ofm_ctx* c);
 // region-stacked contraction (region.cu)
 ofm_status ofm_region_plan(ofm_ctx* c);

@@ -61,15 +61,9 @@ namespace {
 // plane, each plane padded to a multiple of 8 points (p8): point (ix, iy, iz)
 // has K index iz * p8 + iy * L[0] + ix, so a 16-byte operand unit (8 BF16 or
 // 4 TF32 points) never straddles two planes.  K is padded to 64-point tiles.
-struct RUnit {
-  int frag;
-  int s0[3];          // region start (global grid coordinates)
-  int L[3];           // region extent
-  int p8;             // plane stride in K: L[0] * L[1] rounded up to 8
-  int ntiles;         // 64-point tiles: (L[2] * p8) / 64 rounded up
-  long long tile0;    // first global tile of this unit
-  long long base;     // byte offset of the block in the plane arena
-};
+// The pair schedule packs every fragment's storage box once in the same order,
+// its x range widened to whole 8-point units of the grid (tc.cu): RUnit
+// (ofm_internal.h) describes both.
 
 // One contraction work item: up to 256 rows (two 128-row halves sharing the
 // B operand) x an N tile of one region part.
@@ -141,6 +135,10 @@ template <> struct KindT<RK_F32> {
 };
 template <> struct KindT<RK_F64> {
   static constexpr int esz = 8, KC = 16, CPT = 4;
+};
+// pair schedule: a chunk is one 8-point unit
+template <int K> struct PairT : KindT<K> {
+  static constexpr int KC = 8, CPT = 8;
 };
 // byte scale of a kind's plane layout against the plan's offsets (FP64: 2)
 __host__ __device__ constexpr int kind_scale(int k) { return k == RK_F64 ? 2 : 1; }
@@ -227,13 +225,15 @@ __device__ __forceinline__ uint32_t rtf32(float x) {
 // CHECK (check mode): every gathered point index is tested against the
 // fragment's dilated box and the states arena, every 16-byte store against
 // the plane arena; a failing access is skipped and *bounds set.
-template <int KIND, bool CHECK = false>
+// PAIR: chunks of one 8-point unit; gxw is the grid's x extent in whole units
+// times 8 (the points past gx do not exist), gx otherwise.
+template <int KIND, bool CHECK = false, bool PAIR = false>
 __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
     const RUnit* __restrict__ units, const int4* __restrict__ cta, const DevFrag* __restrict__ fr,
     const float* __restrict__ V, const float* __restrict__ states, unsigned char* __restrict__ planes,
-    int gx, int gy, int gz, double c0d, double c1d, long long n_states, long long n_plane_bytes,
+    int gx, int gy, int gz, int gxw, double c0d, double c1d, long long n_states, long long n_plane_bytes,
     int* bounds) {
-  using KT = KindT<KIND>;
+  using KT = typename std::conditional<PAIR, PairT<KIND>, KindT<KIND>>::type;
   constexpr int ESZ = KT::esz;
   constexpr int KPU = 16 / ESZ;            // points per 16-byte unit
   constexpr int NCORE = KT::KC / KPU;      // 16-byte core columns per chunk
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
   const int qpp = F.ld / 4;
   const int nq = rows / 4;
   const int npl = U.L[0] * U.L[1];
-  const long long cb = (long long)rows * 64 * SCL;
+  const long long cb = (long long)rows * KT::KC * ESZ;   // bytes of a K chunk
   const long long npl2 = (long long)U.ntiles * 128 * rows;   // one 2-byte plane
   const long long half = 2 * npl2 * SCL;                     // phi planes -> H phi planes
   const int upc = rows * NCORE;                              // units per chunk and plane
@@ -301,7 +301,12 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         int g = U.s0[d] + ii[d];
-        if (g >= gn[d]) g -= gn[d];
+        const int gw = d == 0 ? gxw : gn[d];
+        if (g >= gw) g -= gw;
+        if (PAIR && g >= gn[d]) {
+          in = false;
+          g = 0;
+        }
         gi[d] = g;
         int ld = g - F.doff[d];
         if (ld < 0) ld += gn[d];
@@ -1677,8 +1682,8 @@ ofm_status ofm_region_run(ofm_ctx* c, ofm_precision prec) {
       int* bd = (int*)c->flag.p + OFM_FLAG_BOUNDS;
 #define OFM_PACK(K, CH)                                                                        \
   pack_kernel<K, CH><<<grid, PK_THREADS, sm, c->stream>>>(u, cta, f, V, st, pl, c->grid.n[0],  \
-                                                         c->grid.n[1], c->grid.n[2], c0, c1, \
-                                                         nst, npb, bd)
+                                                         c->grid.n[1], c->grid.n[2],         \
+                                                         c->grid.n[0], c0, c1, nst, npb, bd)
       const bool ch = c->checks;
       if (kind == RK_TF32) { if (ch) OFM_PACK(RK_TF32, true); else OFM_PACK(RK_TF32, false); }
       else if (kind == RK_BF16) { if (ch) OFM_PACK(RK_BF16, true); else OFM_PACK(RK_BF16, false); }
@@ -1746,6 +1751,50 @@ ofm_status ofm_region_run(ofm_ctx* c, ofm_precision prec) {
     OFM_CUDA(c, cudaGetLastError());
   }
   c->tc_check = kind <= RK_BF16X3;
+  return OFM_OK;
+}
+
+// The operand planes of the pair schedule (tc.cu): shared-memory limits, the
+// arena (the region schedule's, only one of the two is in use at a time) and
+// the launch.  kind: TF32, BF16, BF16 hi+lo.
+ofm_status ofm_pair_planes(ofm_ctx* c, long long bytes, void** arena) {
+  if (!c->region) c->region = new RegionPlan();
+  OFM_TRY(ofm_ensure_big(c, c->region->planes, (size_t)bytes, "operand planes"));
+  *arena = c->region->planes.p;
+  static bool attr = false;
+  if (!attr) {
+    const int pk = 2 * 64 * (RS_MAXROWS + 4) * 4;
+    const void* k[6] = {(const void*)pack_kernel<RK_TF32, false, true>, (const void*)pack_kernel<RK_TF32, true, true>,
+                        (const void*)pack_kernel<RK_BF16, false, true>, (const void*)pack_kernel<RK_BF16, true, true>,
+                        (const void*)pack_kernel<RK_BF16X3, false, true>,
+                        (const void*)pack_kernel<RK_BF16X3, true, true>};
+    for (const void* q : k) cudaFuncSetAttribute(q, cudaFuncAttributeMaxDynamicSharedMemorySize, pk);
+    OFM_CUDA(c, cudaGetLastError());
+    attr = true;
+  }
+  return OFM_OK;
+}
+
+ofm_status ofm_pair_pack(ofm_ctx* c, int kind, const RUnit* units, const int4* cta, int ncta, void* arena,
+                         long long bytes) {
+  KTimer t(c, KC_APPLY, 1, c->pack_bytes[kind]);
+  const double h = c->grid.h, c0 = 3.0 / (h * h), c1 = 0.5 / (h * h);
+  int maxrows = 8;
+  for (const DevFrag& f : c->frags) maxrows = std::max(maxrows, (f.n + 7) / 8 * 8);
+  const int sm = 2 * 64 * ((maxrows + 31) / 32 * 32 + 4) * 4;
+  const int* gn = c->grid.n;
+#define OFM_PACKP(K, CH)                                                                              \
+  pack_kernel<K, CH, true><<<ncta, PK_THREADS, sm, c->stream>>>(                                      \
+      units, cta, (const DevFrag*)c->d_frags.p, (const float*)c->V.p, (const float*)c->states.p,      \
+      (unsigned char*)arena, gn[0], gn[1], gn[2], (gn[0] + 7) / 8 * 8, c0, c1, c->state_elems, bytes, \
+      (int*)c->flag.p + OFM_FLAG_BOUNDS)
+  if (ncta > 0) {
+    if (kind == RK_TF32) { if (c->checks) OFM_PACKP(RK_TF32, true); else OFM_PACKP(RK_TF32, false); }
+    else if (kind == RK_BF16) { if (c->checks) OFM_PACKP(RK_BF16, true); else OFM_PACKP(RK_BF16, false); }
+    else { if (c->checks) OFM_PACKP(RK_BF16X3, true); else OFM_PACKP(RK_BF16X3, false); }
+  }
+#undef OFM_PACKP
+  OFM_CUDA(c, cudaGetLastError());
   return OFM_OK;
 }
 

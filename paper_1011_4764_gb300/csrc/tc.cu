@@ -1,21 +1,32 @@
-// Pair-block contraction on the 5th-generation tensor cores (tcgen05):
+// Pair-block contraction on the 5th-generation tensor cores (tcgen05), the
+// "pair" schedule:
 //     [S_ab | H_ab] = Phi_a[R]^T [Phi_b[R] | HPhi_b[R]]   (Sec. II),
-// M = n_a (padded to 128), N = 2 n_b (padded to a multiple of 16), K = |R|.
+// M = n_a (padded to 128), N = 2 n_b (each half padded to 16), K = |R|.
 //
-// The work is cut into items (pair, rows of a piece); a persistent CTA per SM
-// streams its items through a warp-specialised pipeline (one thread issues
-// bulk copies of the K step's point rows into a ring of raw stages; four
-// warps convert them into the K-major, no-swizzle canonical operand layout
-// of the MMA -- core matrices of 8 rows x 16 bytes, K-adjacent cores 128
-// bytes apart, 8-row groups one K-tile apart -- as TF32 (round to nearest),
-// BF16 (round to nearest even) or the BF16 pair hi = bf16(x),
-// lo = bf16(x - hi); one thread issues tcgen05.mma with FP32 accumulation in
-// tensor memory, hi*hi + hi*lo + lo*hi for the split (lo*lo dropped); four
-// warps read the accumulator with tcgen05.ld and write the item's FP32
-// partial tile).  A finalize kernel sums the partials of each pair in a
-// fixed order.  Every wait is bounded: on timeout the CTA sets an error
-// flag, drains its copies and MMAs, frees its tensor memory and returns.
-#include <cuda_bf16.h>
+// Operands.  pack_kernel (region.cu) writes every fragment's states and H phi
+// once per assembly, over its storage box with the x range widened to whole
+// 8-point units of the grid: unit (x/8, y, z) of a fragment is one contiguous
+// block of rows_pad x 8 points in the K-major no-swizzle operand layout (core
+// matrices of 8 states x 16 bytes; TF32 two cores per 8-state group, BF16 one),
+// phi and H phi as separate planes, BF16 hi and lo too.  Both fragments of a
+// pair share the grid's units and are zero outside their own boxes, so the pair
+// sums over the units that both touch, and a run of units along x is one bulk
+// copy per operand: no conversion stands between the copies and the MMAs.  (The
+// form before converted FP32 rows in shared memory, once per pair a fragment is
+// in, through a transposing read: contraction 2.13 ms and H apply 0.12 ms for 56
+// uneven boxes with 826 pairs, TF32; now 0.58 and, with the operands, 0.24 ms.)
+//
+// A persistent CTA per SM takes items (pair, rows of units of a piece) from a
+// global counter, the largest first, through a warp-specialised pipeline: a
+// producer warp issues the copies of a stage (one run of units per lane), one
+// thread issues the MMAs into two alternating TMEM accumulators (a K step is one
+// unit in TF32, two in BF16; hi*hi + hi*lo + lo*hi for the split), four warps
+// drain an accumulator into the item's FP32 partial tile.  Operand rows past a
+// fragment's own (M to 128, N to 16) are whatever follows in shared memory:
+// they reach only accumulator rows and columns that nobody reads.  A finalize
+// kernel sums the partials of each pair in a fixed order.  Every wait is
+// bounded: on timeout the CTA sets an error flag, drains its copies and MMAs,
+// frees its tensor memory and returns.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -31,27 +42,33 @@ using namespace ofm::ptx;
 
 namespace {
 
+struct TcFrag {
+  int nux, dext1;     // x units and y extent of the storage box
+  int n, rows;        // states, padded to 8
+  long long base;     // byte offset in the plane arena
+  long long npl2;     // bytes of one 2-byte plane: hi -> lo, and half of phi -> H phi
+};
+
 struct TcPair {
   int a, b;
   int item0, nitem;
-  int N, Npad;          // 2 n_b and its padding to a multiple of 16
   long long blk_off;    // block arena offset (same layout as the CUDA-core path)
 };
 
 struct TcItem {
   int pair;
-  int piece;
-  int r0, r1;
-  long long part_off;   // FP32 partial tile of n_a x N
+  int la[3], lb[3];     // start of the piece in both storage boxes (x in units)
+  int m, leny;          // units per row, rows per z plane of the piece
+  int r0, r1;           // rows of the item
+  long long part_off;   // FP32 partial tile of n_a x 2 n_b
 };
 
-
-// operand kinds: TF32, BF16, BF16 hi+lo, TF32 hi+lo (the last for FP32-class
-// Gram matrices: hi = tf32(x), lo = tf32(x - hi), products to about 2^-22)
-enum { TC_TF32 = 0, TC_BF16 = 1, TC_BF16X3 = 2, TC_TF32X3 = 3, TC_NKIND = 4 };
-
-template <int KIND> constexpr bool is_tf32() { return KIND == TC_TF32 || KIND == TC_TF32X3; }
-template <int KIND> constexpr bool is_split() { return KIND == TC_BF16X3 || KIND == TC_TF32X3; }
+enum { TC_TF32 = 0, TC_BF16 = 1, TC_BF16X3 = 2, TC_NKIND = 3 };
+template <int KIND> struct TcKind {
+  static constexpr int UB = KIND == TC_TF32 ? 32 : 16;   // bytes of a unit per state
+  static constexpr int NPL = KIND == TC_BF16X3 ? 2 : 1;  // planes per operand
+  static constexpr int KU = KIND == TC_TF32 ? 1 : 2;     // units per MMA
+};
 
 // ----------------------------------------------------------- PTX helpers --
 
@@ -83,7 +100,7 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t fmt, uint32_t M, uint
 template <int KIND>
 __device__ __forceinline__ void mma(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                     uint32_t accum) {
-  if constexpr (is_tf32<KIND>()) {
+  if constexpr (KIND == TC_TF32) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
@@ -116,108 +133,65 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ uint32_t f32_to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return r;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-
 // ----------------------------------------------------------- the kernel ---
 
-// Fixed per plan: the largest row strides (floats), operand tile rows,
-// ring sizes and tile bytes.
-struct SmemLayout {
-  int ldA, ldB;        // raw row strides (floats), the largest of the plan
-  int Rb;              // B tile rows (largest Npad)
-  int kt;              // grid points per K step (operand stage): 64, or 32 where 64 does not fit
-  int raw_stage;       // bytes of one raw stage: rsteps x kt points x (ldA + 2 ldB) floats
-  int nraw;            // raw stages in the ring
-  int nop;             // operand stages in the ring (2..TS_NOP)
-  int rsteps;          // K steps per raw stage
-  int tileA, tileB;    // bytes of one operand tile
-  int ntiles;          // operand tiles per operand (1, or 2 for hi+lo)
-  int nitems;          // work items of the plan
-};
+constexpr int TS_THREADS = 192;       // warp 0 copies, 1 MMA, 2-5 epilogue
+constexpr int TS_NSTAGE = 4;
+constexpr int TS_STAGE = 48 * 1024;
+constexpr int TS_UMAX = 32;           // units of a stage at most (one run per lane)
+constexpr int TS_NQ = 4;              // work-item ring between the roles
+constexpr int TS_ACC_COLS = 256;      // TMEM columns of one accumulator; two of them
+// stages, then room for the operand rows read past the last one, then 2 KB of
+// zeros (the second half of a BF16 K step whose item ends with a single unit)
+constexpr int TS_SLACK = 8 * 1024, TS_ZERO = TS_NSTAGE * TS_STAGE + TS_SLACK, TS_SMEM = TS_ZERO + 2048;
 
-constexpr int TS_THREADS = 448;  // warp 0 copies, 1 MMA, 2-9 convert, 10-13 epilogue
-constexpr int TS_NOP = 4;        // largest operand ring
-constexpr int TS_CONV = 8;       // converter warps
-constexpr int TS_MAXRAW = 8;
-constexpr int TS_ACC_COLS = 256; // columns of one accumulator (N <= 256); two of them
+// Units per stage of a pair: a stage holds the units of both operands' planes;
+// even, so that only an item's last stage can end with half a BF16 K step.
+constexpr int TS_MINUNITS = 256;       // units an item may take whatever part of them is padding
+template <int KIND>
+__host__ __device__ constexpr int tc_units(int ra, int rb) {
+  const int u = TS_STAGE / ((ra + 2 * rb) * TcKind<KIND>::UB * TcKind<KIND>::NPL);
+  return u > TS_UMAX ? TS_UMAX : u / 2 * 2;
+}
+static_assert(tc_units<TC_TF32>(128, 128) >= 2 && tc_units<TC_BF16X3>(128, 128) >= 2, "two units fit a stage");
 
-// Persistent, warp-specialised contraction: CTA c takes items c, c + grid,
-// c + 2 grid, ...; every role walks the same item sequence, so a global step
-// counter g indexes the rings.
-//   warp 0   : its lanes issue bulk copies of the K step's point rows (a
-//              contiguous x-run of a piece is contiguous in both fragments'
-//              storage: one copy per run and operand, one run per lane) into
-//              raw stage g % nraw;
-//   warps 2-9: convert raw stage -> operand stage g % nop (canonical K-major
-//              layout, TF32 / BF16 / BF16 hi+lo), zero past the item's end;
-//   warp 1   : one thread issues the MMAs of the stage into the item's
-//              accumulator (two in tensor memory, alternating per item) and
-//              commits them to the stage's "empty" barrier, and after the
-//              item's last stage to the accumulator's "full" barrier;
-//   warps 10-13: read the accumulator (warp w owns lanes 32 (w % 4)..), write
-//              the item's FP32 partial tile, release the accumulator.
-// mbarriers: raw full (copy bytes) / empty (8 converter warps), operand
-// full (8 converter warps) / empty (MMA commit), accumulator full (MMA
-// commit) / empty (4 epilogue warps).  Every wait is bounded and also stops
-// when another role gave up; the CTA then waits (bounded) for its copies and
-// MMAs in flight, frees its tensor memory and returns.
-template <int KIND, int KT>
+template <int KIND>
 __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
-    const DevFrag* __restrict__ fr, const TcPair* __restrict__ prs, const Piece* __restrict__ pcs,
-    const TcItem* __restrict__ items, const float* __restrict__ states,
-    const float* __restrict__ hphi, float* __restrict__ partials, int* flag, SmemLayout L) {
+    const TcFrag* __restrict__ fr, const TcPair* __restrict__ prs, const TcItem* __restrict__ items,
+    const int* __restrict__ order, int nitems, const unsigned char* __restrict__ planes,
+    float* __restrict__ partials, int* flag, int* next) {
+  using KT = TcKind<KIND>;
+  constexpr int UB = KT::UB, NPL = KT::NPL, KU = KT::KU;
+  constexpr uint32_t SBO = 8 * UB;     // next 8-state group of a unit
   extern __shared__ __align__(1024) unsigned char smem[];
-  __shared__ __align__(8) unsigned long long raw_full[TS_MAXRAW], raw_empty[TS_MAXRAW];
-  __shared__ __align__(8) unsigned long long op_full[TS_NOP], op_empty[TS_NOP], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) unsigned long long full[TS_NSTAGE], empty[TS_NSTAGE], acc_full[2], acc_empty[2];
+  __shared__ __align__(8) unsigned long long q_full[TS_NQ], q_empty[TS_NQ];
+  __shared__ int q_item[TS_NQ];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_s, issued_s, mma_steps_s;
-
-  constexpr int ESZ = is_tf32<KIND>() ? 4 : 2;
-  constexpr int E = 16 / ESZ;                 // elements per core row
-  constexpr uint32_t LBO = 128;               // K-adjacent cores
-  constexpr uint32_t SBO = (KT / E) * 128;    // next 8-row group
-  constexpr int KSTEPS = (KT * ESZ) / 32;     // MMAs per K step (32 bytes of K each)
-  constexpr int NG = KT / E;                  // core groups along K
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nraw = L.nraw, nop = L.nop;
-  const int span = L.rsteps * KT;   // points per raw stage
-  unsigned char* raw = smem;
-  unsigned char* ops = smem + (size_t)nraw * L.raw_stage;
-  auto tileA = [&](int o, int t) {
-    return ops + (size_t)o * L.ntiles * (L.tileA + L.tileB) + (size_t)t * L.tileA;
-  };
-  auto tileB = [&](int o, int t) {
-    return ops + (size_t)o * L.ntiles * (L.tileA + L.tileB) + (size_t)L.ntiles * L.tileA +
-           (size_t)t * L.tileB;
-  };
 
   if (tid == 0) {
-    for (int i = 0; i < nraw; ++i) {
-      mbar_init(smem_u32(&raw_full[i]), 1);
-      mbar_init(smem_u32(&raw_empty[i]), TS_CONV);
-    }
-    for (int i = 0; i < L.nop; ++i) {
-      mbar_init(smem_u32(&op_full[i]), TS_CONV);
-      mbar_init(smem_u32(&op_empty[i]), 1);
+    for (int i = 0; i < TS_NSTAGE; ++i) {
+      mbar_init(smem_u32(&full[i]), 1);
+      mbar_init(smem_u32(&empty[i]), 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&acc_full[i]), 1);
       mbar_init(smem_u32(&acc_empty[i]), 4);
+    }
+    for (int i = 0; i < TS_NQ; ++i) {
+      mbar_init(smem_u32(&q_full[i]), 1);
+      mbar_init(smem_u32(&q_empty[i]), 5);   // the MMA thread and the four epilogue warps
     }
     fence_mbar_init();
     abort_s = 0;
     issued_s = 0;
     mma_steps_s = 0;
   }
+  for (int i = tid; i < 2048 / 16; i += TS_THREADS)
+    reinterpret_cast<uint4*>(smem + TS_ZERO)[i] = make_uint4(0, 0, 0, 0);
+  fence_async_smem();   // the zeros are read by the tensor cores
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
@@ -241,229 +215,168 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
     *(volatile int*)&abort_s = 1;
     return false;
   };
-  const int nitems = L.nitems;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ copies
-    // one raw stage holds `span` points of the item (rsteps K steps); lane j
-    // issues the copies of runs j, j + 32, ...: run 0 starts at the stage's
-    // first point, run i > 0 at the start of the i-th following row
-    int gr = 0;
+    // ---------------------------------------------------------- producer
+    int g = 0;
     bool ok = true;
-    for (int ii = blockIdx.x; ii < nitems && ok; ii += gridDim.x) {
+    for (int item_no = 0; ok; ++item_no) {
+      const int qs = item_no % TS_NQ, qu = item_no / TS_NQ;
+      int ii = 0;
+      if (lane == 0) {
+        const bool w = qu == 0 || wait(&q_empty[qs], (uint32_t)((qu - 1) & 1));
+        ii = w ? atomicAdd(next, 1) : nitems;
+        ii = ii < nitems ? order[ii] : -1;
+        q_item[qs] = ii;
+        mbar_arrive(smem_u32(&q_full[qs]));   // release: the index is visible to the waiters
+        ok = w;
+      }
+      ii = __shfl_sync(0xffffffffu, ii, 0);
+      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      if (!ok || ii < 0) break;
       const TcItem it = items[ii];
       const TcPair pr = prs[it.pair];
-      const DevFrag A = fr[pr.a], B = fr[pr.b];
-      const Piece pc = pcs[it.piece];
-      const int lenx = pc.len[0], leny = pc.len[1];
-      const int npts = (it.r1 - it.r0) * lenx;
-      for (int k0 = 0; k0 < npts; k0 += span, ++gr) {
-        const int s = gr % nraw, u = gr / nraw;
-        if (u > 0) {   // lane 0 waits; the outcome is the warp's (uniform control flow)
+      const TcFrag A = fr[pr.a], B = fr[pr.b];
+      const int ua = A.rows * UB, ub = B.rows * UB;
+      const int U = tc_units<KIND>(A.rows, B.rows);
+      const int nu = (it.r1 - it.r0) * it.m;
+      for (int k0 = 0; k0 < nu; k0 += U, ++g) {
+        const int s = g % TS_NSTAGE, u = g / TS_NSTAGE;
+        if (u > 0) {
           bool w = true;
-          if (lane == 0) w = wait(&raw_empty[s], (uint32_t)((u - 1) & 1));
+          if (lane == 0) w = wait(&empty[s], (uint32_t)((u - 1) & 1));
           ok = __shfl_sync(0xffffffffu, w ? 1 : 0, 0) != 0;
           if (!ok) break;
         }
-        const int nk = min(span, npts - k0);
-        const uint32_t mb = smem_u32(&raw_full[s]);
-        if (lane == 0) mbar_arrive_expect(mb, (uint32_t)(nk * (A.ld + 2 * B.ld) * 4));
+        const int nk = min(U, nu - k0);
+        const uint32_t mb = smem_u32(&full[s]);
+        if (lane == 0) mbar_arrive_expect(mb, (uint32_t)(nk * (ua + 2 * ub) * NPL));
         __syncwarp();
-        const int row0 = k0 / lenx, x0 = k0 - row0 * lenx;
-        const int nruns = (k0 + nk - 1) / lenx - row0 + 1;   // <= span
-        unsigned char* rA = raw + (size_t)s * L.raw_stage;
-        unsigned char* rB = rA + (size_t)span * L.ldA * 4;
-        unsigned char* rH = rB + (size_t)span * L.ldB * 4;
-        for (int j = lane; j < nruns; j += 32) {
-          const int x = j == 0 ? x0 : 0;
-          const int kstart = j == 0 ? k0 : (row0 + j) * lenx;
-          const int run = min(lenx - x, k0 + nk - kstart);
-          const int r = it.r0 + row0 + j;
-          const int y = r % leny, z = r / leny;
-          const long long pa =
-              ((long long)(pc.la[2] + z) * A.dext[1] + (pc.la[1] + y)) * A.dext[0] + pc.la[0] + x;
-          const long long pb =
-              ((long long)(pc.lb[2] + z) * B.dext[1] + (pc.lb[1] + y)) * B.dext[0] + pc.lb[0] + x;
-          const int kk = kstart - k0;
-          bulk_g2s(smem_u32(rA + (size_t)kk * A.ld * 4), states + A.off + pa * A.ld,
-                   (uint32_t)(run * A.ld * 4), mb);
-          bulk_g2s(smem_u32(rB + (size_t)kk * B.ld * 4), states + B.off + pb * B.ld,
-                   (uint32_t)(run * B.ld * 4), mb);
-          bulk_g2s(smem_u32(rH + (size_t)kk * B.ld * 4), hphi + B.off + pb * B.ld,
-                   (uint32_t)(run * B.ld * 4), mb);
+        const int row0 = k0 / it.m, x0 = k0 - row0 * it.m;
+        const int nruns = (k0 + nk - 1) / it.m - row0 + 1;   // <= U <= 32
+        if (lane < nruns) {
+          const int x = lane == 0 ? x0 : 0;
+          const int ks = lane == 0 ? k0 : (row0 + lane) * it.m;
+          const int run = min(it.m - x, k0 + nk - ks);
+          const int r = it.r0 + row0 + lane;
+          const int y = r % it.leny, z = r / it.leny;
+          const long long qa = ((long long)(it.la[2] + z) * A.dext1 + it.la[1] + y) * A.nux + it.la[0] + x;
+          const long long qb = ((long long)(it.lb[2] + z) * B.dext1 + it.lb[1] + y) * B.nux + it.lb[0] + x;
+          const unsigned char* sa = planes + A.base + qa * ua;
+          const unsigned char* sb = planes + B.base + qb * ub;
+          const uint32_t d = smem_u32(smem + (size_t)s * TS_STAGE);
+          const uint32_t dB = d + (uint32_t)(NPL * U * ua), dH = dB + (uint32_t)(NPL * U * ub);
+          const uint32_t oa = (uint32_t)((ks - k0) * ua), ob = (uint32_t)((ks - k0) * ub);
+#pragma unroll
+          for (int pl = 0; pl < NPL; ++pl) {
+            bulk_g2s(d + (uint32_t)(pl * U * ua) + oa, sa + pl * A.npl2, (uint32_t)(run * ua), mb);
+            bulk_g2s(dB + (uint32_t)(pl * U * ub) + ob, sb + pl * B.npl2, (uint32_t)(run * ub), mb);
+            bulk_g2s(dH + (uint32_t)(pl * U * ub) + ob, sb + (2 + pl) * B.npl2, (uint32_t)(run * ub), mb);
+          }
         }
-        if (lane == 0) *(volatile int*)&issued_s = gr + 1;
+        if (lane == 0) *(volatile int*)&issued_s = g + 1;
       }
     }
   } else if (warp == 1) {
     // -------------------------------------------------------------- MMAs
     if (lane == 0) {
-      constexpr uint32_t FMT = is_tf32<KIND>() ? 2u : 1u;
-      int g = 0, item_no = 0;
+      constexpr uint32_t FMT = KIND == TC_TF32 ? 2u : 1u;
+      int g = 0;
       bool ok = true;
-      for (int ii = blockIdx.x; ii < nitems && ok; ii += gridDim.x, ++item_no) {
+      for (int item_no = 0; ok; ++item_no) {
+        const int qs = item_no % TS_NQ, qu = item_no / TS_NQ;
+        if (!(ok = wait(&q_full[qs], (uint32_t)(qu & 1)))) break;
+        const int ii = *(volatile int*)&q_item[qs];
+        mbar_arrive(smem_u32(&q_empty[qs]));
+        if (ii < 0) break;
         const TcItem it = items[ii];
         const TcPair pr = prs[it.pair];
-        const Piece pc = pcs[it.piece];
-        const int npts = (it.r1 - it.r0) * pc.len[0];
-        const int b = item_no & 1, ub = item_no >> 1;
-        if (ub > 0 && !(ok = wait(&acc_empty[b], (uint32_t)((ub - 1) & 1)))) break;
+        const int ra = fr[pr.a].rows, rb = fr[pr.b].rows;
+        const int ua = ra * UB, ub = rb * UB, U = tc_units<KIND>(ra, rb);
+        const int nu = (it.r1 - it.r0) * it.m;
+        const uint32_t N = (uint32_t)((rb + 15) / 16 * 16);
+        const uint32_t idesc = instr_desc(FMT, 128, N);
+        const int b = item_no & 1, ubar = item_no >> 1;
+        if (ubar > 0 && !(ok = wait(&acc_empty[b], (uint32_t)((ubar - 1) & 1)))) break;
         tc_fence_after();
-        const uint32_t idesc = instr_desc(FMT, 128, (uint32_t)pr.Npad);
-        const uint32_t dacc = tmem + (uint32_t)(b * TS_ACC_COLS);
-        for (int k0 = 0; k0 < npts; k0 += KT, ++g) {
-          const int o = g % nop, uo = g / nop;
-          if (!(ok = wait(&op_full[o], (uint32_t)(uo & 1)))) break;
+        const uint32_t dS = tmem + (uint32_t)(b * TS_ACC_COLS), dH = dS + N;
+        for (int k0 = 0; k0 < nu; k0 += U, ++g) {
+          const int s = g % TS_NSTAGE, u = g / TS_NSTAGE;
+          if (!(ok = wait(&full[s], (uint32_t)(u & 1)))) break;
           tc_fence_after();
-          // descriptors of the stage's tiles; a K sub-step advances the
-          // start address by two core matrices (the field holds address >> 4)
-          const uint64_t ah0 = smem_desc(smem_u32(tileA(o, 0)), LBO, SBO);
-          const uint64_t bh0 = smem_desc(smem_u32(tileB(o, 0)), LBO, SBO);
-          uint64_t al0 = 0, bl0 = 0;
-          if constexpr (is_split<KIND>()) {
-            al0 = smem_desc(smem_u32(tileA(o, 1)), LBO, SBO);
-            bl0 = smem_desc(smem_u32(tileB(o, 1)), LBO, SBO);
-          }
-#pragma unroll
-          for (int ks = 0; ks < KSTEPS; ++ks) {
-            const uint64_t off = (uint64_t)((ks * 2 * LBO) >> 4);
-            mma<KIND>(dacc, ah0 + off, bh0 + off, idesc, (k0 > 0 || ks > 0) ? 1u : 0u);
-            if constexpr (is_split<KIND>()) {
-              mma<KIND>(dacc, ah0 + off, bl0 + off, idesc, 1u);
-              mma<KIND>(dacc, al0 + off, bh0 + off, idesc, 1u);
+          const int nk = min(U, nu - k0);
+          const uint32_t zero = smem_u32(smem + TS_ZERO);
+          uint32_t a = smem_u32(smem + (size_t)s * TS_STAGE);
+          uint32_t p = a + (uint32_t)(NPL * U * ua), h = p + (uint32_t)(NPL * U * ub);
+          const uint32_t la = (uint32_t)(U * ua), lb = (uint32_t)(U * ub);   // hi -> lo
+          for (int q = 0; q < nk; q += KU) {
+            // TF32: both cores of the unit; BF16: this unit's core and the next
+            // unit's (zeros after the last)
+            const bool two = KU == 1 || q + 1 < nk;
+            auto desc = [&](uint32_t addr, uint32_t ustep) {
+              return smem_desc(addr, KU == 1 ? 128u : two ? ustep : zero - addr, SBO);
+            };
+            const uint64_t a0 = desc(a, (uint32_t)ua), p0 = desc(p, (uint32_t)ub), h0 = desc(h, (uint32_t)ub);
+            const uint32_t acc = (k0 > 0 || q > 0) ? 1u : 0u;
+            mma<KIND>(dS, a0, p0, idesc, acc);
+            mma<KIND>(dH, a0, h0, idesc, acc);
+            if constexpr (NPL == 2) {
+              const uint64_t a1 = desc(a + la, (uint32_t)ua), p1 = desc(p + lb, (uint32_t)ub),
+                             h1 = desc(h + lb, (uint32_t)ub);
+              mma<KIND>(dS, a0, p1, idesc, 1u);
+              mma<KIND>(dH, a0, h1, idesc, 1u);
+              mma<KIND>(dS, a1, p0, idesc, 1u);
+              mma<KIND>(dH, a1, h0, idesc, 1u);
             }
+            a += (uint32_t)(KU * ua);
+            p += (uint32_t)(KU * ub);
+            h += (uint32_t)(KU * ub);
           }
-          mma_commit(smem_u32(&op_empty[o]));
+          mma_commit(smem_u32(&empty[s]));
           *(volatile int*)&mma_steps_s = g + 1;
         }
         if (!ok) break;
         mma_commit(smem_u32(&acc_full[b]));
       }
     }
-  } else if (warp < 2 + TS_CONV) {
-    // -------------------------------------------------------- conversion
-    const int ct = tid - 64;   // 0 .. 32 TS_CONV - 1
-    int gr = 0, go = 0;
-    bool ok = true;
-    for (int ii = blockIdx.x; ii < nitems && ok; ii += gridDim.x) {
-      const TcItem it = items[ii];
-      const TcPair pr = prs[it.pair];
-      const DevFrag A = fr[pr.a], B = fr[pr.b];
-      const Piece pc = pcs[it.piece];
-      const int npts = (it.r1 - it.r0) * pc.len[0];
-      const int N = pr.N;
-      // e -> (row, k group) without integer division: e / rows from a float
-      // reciprocal, corrected by one (exact for e < 2^24)
-      const float inv_a = 1.0f / (float)A.n, inv_n = 1.0f / (float)N;
-      for (int k0 = 0; k0 < npts && ok; k0 += span, ++gr) {
-        const int s = gr % nraw, u = gr / nraw;
-        // every lane waits (it reads the copied data); the outcome is the warp's
-        ok = __all_sync(0xffffffffu, wait(&raw_full[s], (uint32_t)(u & 1)));
-        if (!ok) break;
-        const int nkr = min(span, npts - k0);
-        const float* rA = reinterpret_cast<const float*>(raw + (size_t)s * L.raw_stage);
-        const float* rB = rA + (size_t)span * L.ldA;
-        const float* rH = rB + (size_t)span * L.ldB;
-        for (int j0 = 0; j0 < nkr; j0 += KT, ++go) {
-          const int o = go % nop, uo = go / nop;
-          if (uo > 0) {
-            ok = __all_sync(0xffffffffu, wait(&op_empty[o], (uint32_t)((uo - 1) & 1)));
-            if (!ok) break;
-          }
-          const int nk = min(KT, nkr - j0);
-          // operand rows: A = states of fragment a; B = columns 0..n_b-1 from
-          // Phi_b, n_b..2n_b-1 from H Phi_b
-          for (int e = ct; e < (A.n + N) * NG; e += 32 * TS_CONV) {
-            const bool isA = e < A.n * NG;
-            const int e2 = isA ? e : e - A.n * NG;
-            const int rows = isA ? A.n : N;
-            int gq = (int)((float)e2 * (isA ? inv_a : inv_n));
-            if (gq * rows > e2) --gq;
-            else if ((gq + 1) * rows <= e2) ++gq;
-            const int row = e2 - gq * rows;
-            const float* src;
-            int col, ld;
-            if (isA) {
-              src = rA;
-              col = row;
-              ld = A.ld;
-            } else {
-              const bool h = row >= B.n;
-              src = h ? rH : rB;
-              col = h ? row - B.n : row;
-              ld = B.ld;
-            }
-            src += (size_t)j0 * ld + col;
-            float v[E];
-#pragma unroll
-            for (int j = 0; j < E; ++j) {
-              const int kk = gq * E + j;
-              v[j] = kk < nk ? src[kk * ld] : 0.f;
-            }
-            const size_t off = (size_t)(row >> 3) * SBO + (size_t)gq * LBO + (size_t)(row & 7) * 16;
-            unsigned char* t0 = isA ? tileA(o, 0) : tileB(o, 0);
-            if constexpr (is_tf32<KIND>()) {
-              uint32_t hi[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) hi[j] = f32_to_tf32(v[j]);
-              *reinterpret_cast<uint4*>(t0 + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-              if constexpr (KIND == TC_TF32X3) {
-                uint32_t lo[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) lo[j] = f32_to_tf32(v[j] - __uint_as_float(hi[j]));
-                unsigned char* t1 = isA ? tileA(o, 1) : tileB(o, 1);
-                *reinterpret_cast<uint4*>(t1 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-              }
-            } else {
-              uint32_t hi[4], lo[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                hi[j] = pack_bf16(v[2 * j], v[2 * j + 1]);
-                if constexpr (KIND == TC_BF16X3) {
-                  __nv_bfloat162 hh = *reinterpret_cast<__nv_bfloat162*>(&hi[j]);
-                  const float2 hf = __bfloat1622float2(hh);
-                  lo[j] = pack_bf16(v[2 * j] - hf.x, v[2 * j + 1] - hf.y);
-                }
-              }
-              *reinterpret_cast<uint4*>(t0 + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-              if constexpr (KIND == TC_BF16X3) {
-                unsigned char* t1 = isA ? tileA(o, 1) : tileB(o, 1);
-                *reinterpret_cast<uint4*>(t1 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-              }
-            }
-          }
-          fence_async_smem();   // generic-proxy writes -> tensor-core reads
-          __syncwarp();
-          if (lane == 0) mbar_arrive(smem_u32(&op_full[o]));
-        }
-        if (!ok) break;
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&raw_empty[s]));   // every K step of the stage read
-      }
-    }
   } else {
     // ---------------------------------------------------------- epilogue
     const int q = warp & 3;   // tensor-memory lane quadrant of this warp
-    int item_no = 0;
     bool ok = true;
-    for (int ii = blockIdx.x; ii < nitems && ok; ii += gridDim.x, ++item_no) {
+    for (int item_no = 0; ok; ++item_no) {
+      const int qs = item_no % TS_NQ, qu = item_no / TS_NQ;
+      ok = __all_sync(0xffffffffu, wait(&q_full[qs], (uint32_t)(qu & 1)));
+      if (!ok) break;
+      const int ii = *(volatile int*)&q_item[qs];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&q_empty[qs]));
+      if (ii < 0) break;
       const TcItem it = items[ii];
       const TcPair pr = prs[it.pair];
-      const int na = fr[pr.a].n, N = pr.N, Npad = pr.Npad;
-      const int b = item_no & 1, ub = item_no >> 1;
-      ok = __all_sync(0xffffffffu, wait(&acc_full[b], (uint32_t)(ub & 1)));
+      const int na = fr[pr.a].n, nb = fr[pr.b].n, N = (fr[pr.b].rows + 15) / 16 * 16;
+      const int b = item_no & 1, ubar = item_no >> 1;
+      ok = __all_sync(0xffffffffu, wait(&acc_full[b], (uint32_t)(ubar & 1)));
       if (!ok) break;
       tc_fence_after();
-      float* out = partials + it.part_off;
       const int row = q * 32 + lane;
-      for (int c0 = 0; c0 < Npad; c0 += 8) {
-        float v[8];
-        tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TS_ACC_COLS + c0), v);
-        if (row < na) {
+      float* out = partials + it.part_off + (long long)row * 2 * nb;
+      if (q * 32 < na) {
+        for (int hf = 0; hf < 2; ++hf)
+          for (int c0 = 0; c0 < nb; c0 += 8) {
+            float v[8];
+            tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TS_ACC_COLS + hf * N + c0), v);
+            if (row < na) {
+              float* o = out + hf * nb + c0;
+              if (c0 + 8 <= nb && (reinterpret_cast<uintptr_t>(o) & 15) == 0) {
+                *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+                *reinterpret_cast<float4*>(o + 4) = make_float4(v[4], v[5], v[6], v[7]);
+              } else {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (c0 + j < N) out[(long long)row * N + c0 + j] = v[j];
-        }
+                for (int j = 0; j < 8; ++j)
+                  if (c0 + j < nb) o[j] = v[j];
+              }
+            }
+          }
       }
       tc_fence_before();
       __syncwarp();
@@ -481,10 +394,10 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
         if (i > 64) __nanosleep(64);
     };
     const int issued = issued_s;
-    for (int g = max(0, issued - nraw); g < issued; ++g)
-      drain(&raw_full[g % nraw], (uint32_t)((g / nraw) & 1));
+    for (int g = max(0, issued - TS_NSTAGE); g < issued; ++g)
+      drain(&full[g % TS_NSTAGE], (uint32_t)((g / TS_NSTAGE) & 1));
     const int ms = mma_steps_s;
-    if (ms > 0) drain(&op_empty[(ms - 1) % nop], (uint32_t)(((ms - 1) / nop) & 1));
+    if (ms > 0) drain(&empty[(ms - 1) % TS_NSTAGE], (uint32_t)(((ms - 1) / TS_NSTAGE) & 1));
   }
   tc_fence_before();
   __syncthreads();
@@ -495,20 +408,34 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
 }
 
 // Sum of the partial tiles of each pair in plan order -> FP64 blocks
-// (H_ab then S_ab, n_a x n_b row-major); diagonal blocks symmetrised.
-__global__ void tc_finalize_kernel(const DevFrag* __restrict__ fr, const TcPair* __restrict__ prs,
-                                   const TcItem* __restrict__ items,
-                                   const float* __restrict__ partials, double* __restrict__ blocks) {
+// (H_ab then S_ab, n_a x n_b row-major); diagonal blocks symmetrised.  A pair's
+// partial tiles are consecutive; the FP32 terms are summed error-free (the
+// rounding error of every addition carried in a second word), without FP64
+// arithmetic per term.
+__global__ void __launch_bounds__(256) tc_finalize_kernel(const TcFrag* __restrict__ fr,
+                                                          const TcPair* __restrict__ prs,
+                                                          const TcItem* __restrict__ items,
+                                                          const float* __restrict__ partials,
+                                                          double* __restrict__ blocks) {
   const TcPair pr = prs[blockIdx.x];
-  const int na = fr[pr.a].n, nb = fr[pr.b].n, N = pr.N;
+  const int na = fr[pr.a].n, nb = fr[pr.b].n, N = 2 * nb;
   double* Hblk = blocks + pr.blk_off;
   double* Sblk = Hblk + (long long)na * nb;
+  const float* base = pr.nitem > 0 ? partials + items[pr.item0].part_off : partials;
+  const long long step = (long long)na * N;
   auto sum = [&](int i, int c) {
-    double s = 0.0;
-    for (int k = 0; k < pr.nitem; ++k) s += (double)partials[items[pr.item0 + k].part_off + (long long)i * N + c];
-    return s;
+    const float* p = base + (long long)i * N + c;
+    float s = 0.f, e = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < pr.nitem; ++k) {
+      const float x = p[k * step];
+      const float t = s + x, bp = t - s;
+      e += (s - (t - bp)) + (x - bp);
+      s = t;
+    }
+    return (double)s + (double)e;
   };
-  // blockIdx.y: a chunk of outputs (the FP64 sums spread over many SMs)
+  // blockIdx.y: a chunk of outputs
   for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < na * nb; e += gridDim.y * blockDim.x) {
     const int i = e / nb, m = e % nb;
     double s = sum(i, m), h = sum(i, nb + m);
@@ -521,32 +448,48 @@ __global__ void tc_finalize_kernel(const DevFrag* __restrict__ fr, const TcPair*
   }
 }
 
+// First unit and number of units (cyclic, NU units of 8 points) that the points
+// [s, s + len) of a periodic axis of n points touch.
+void unit_range(int n, int NU, int s, int len, int& us, int& cnt) {
+  us = s / 8;
+  if (len >= n) {
+    cnt = NU;
+    return;
+  }
+  const int e = s + len - 1;   // < 2 n
+  cnt = e < n ? e / 8 - us + 1 : NU - us + (e - n) / 8 + 1;
+  cnt = std::min(cnt, NU);
+}
+
 }  // namespace
 
 struct TcPlan {
+  std::vector<TcFrag> frags;
+  std::vector<RUnit> units;
+  std::vector<int4> pack_cta;
   std::vector<TcPair> pairs;
   std::vector<TcItem> items;
-  std::vector<Piece> pieces;
-  long long part_elems = 0;
-  SmemLayout lay[TC_NKIND];
-  size_t smem[TC_NKIND] = {0, 0, 0, 0};
-  DevBuf d_pairs, d_items, d_pieces, partials;
-  bool ok = false;
+  std::vector<int> order;       // items, the largest first
+  long long part_elems = 0, plane_bytes = 0;
+  DevBuf d_frags, d_units, d_pcta, d_pairs, d_items, d_order, partials;
+  bool ok = false, uploaded = false;
   std::string why;
 };
 
 void ofm_tc_guards(const TcPlan* t, std::vector<GuardRef>& out) {
   if (!t) return;
   const struct { const DevBuf* b; const char* n; } bufs[] = {
-      {&t->d_pairs, "tensor-core pairs"}, {&t->d_items, "tensor-core items"},
-      {&t->d_pieces, "tensor-core pieces"}, {&t->partials, "tensor-core partials"}};
+      {&t->d_frags, "tensor-core fragments"}, {&t->d_units, "tensor-core pack units"},
+      {&t->d_pcta, "tensor-core pack table"}, {&t->d_pairs, "tensor-core pairs"},
+      {&t->d_items, "tensor-core items"}, {&t->d_order, "tensor-core item order"},
+      {&t->partials, "tensor-core partials"}};
   for (const auto& x : bufs)
     if (x.b->p) out.push_back({x.b->p, x.b->cap, x.n});
 }
 
 void ofm_tc_plan_free(TcPlan* t) {
   if (!t) return;
-  DevBuf* bufs[] = {&t->d_pairs, &t->d_items, &t->d_pieces, &t->partials};
+  DevBuf* bufs[] = {&t->d_frags, &t->d_units, &t->d_pcta, &t->d_pairs, &t->d_items, &t->d_order, &t->partials};
   for (DevBuf* b : bufs)
     if (b->p) cudaFree(b->p);
   delete t;
@@ -557,199 +500,193 @@ void ofm_tc_free(ofm_ctx* c) {
   c->tc = nullptr;
 }
 
-bool ofm_tc_plan_ok(const TcPlan* t, int kind) {
-  return t && t->ok && kind >= 0 && kind < TC_NKIND && t->lay[kind].nraw >= 2;
-}
-
-template <int KIND, int KTT>
-static void set_smem_attr() {
-  cudaFuncSetAttribute(tc_contract_kernel<KIND, KTT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       216 * 1024);
-}
-
-// Tensor-core plan for the pairs over the fragment table fr (FP32 storage,
-// row strides fr[].ld): one item per row chunk of a piece, chunks of about
-// `chunk` points (0: sized for about four items per SM); blk_off[p] is pair
-// p's offset in the FP64 block
-// arena.  The plan is marked not usable (with the reason) when a fragment
-// has more than 128 states or the staging does not fit shared memory.
-ofm_status ofm_tc_plan_build(ofm_ctx* c, TcPlan** tp, const std::vector<DevFrag>& fr,
-                             const std::vector<HostPair>& prs, const std::vector<long long>& blk_off,
-                             long long kh, long long chunk) {
-  if (!*tp) *tp = new TcPlan();
-  TcPlan* t = *tp;
-  t->pairs.clear();
-  t->items.clear();
-  t->pieces.clear();
-  t->part_elems = 0;
-  t->ok = false;
-  int ldA = 4, ldB = 4, Rb = 16;
-  for (const HostPair& hp : prs) {
-    const DevFrag& A = fr[hp.a];
-    const DevFrag& B = fr[hp.b];
-    if (A.n > 128 || 2 * B.n > 256) {
+// Host plan of the pair contraction after a build: one item per row chunk of a
+// piece, chunks of about asm_chunk points (0: sized for about four items per
+// SM).  Not usable (with the reason) for FP64 storage or more than 128 states.
+ofm_status ofm_plan_extra(ofm_ctx* c) {
+  if (!c->tc) c->tc = new TcPlan();
+  TcPlan* t = c->tc;
+  t->frags.clear(); t->units.clear(); t->pack_cta.clear(); t->pairs.clear(); t->items.clear(); t->order.clear();
+  t->part_elems = t->plane_bytes = 0;
+  t->ok = t->uploaded = false;
+  if (c->storage != OFM_STORE_FP32) {
+    t->why = "tensor-core contraction needs FP32 storage";
+    return OFM_OK;
+  }
+  const int n0 = c->grid.n[0], NU = (n0 + 7) / 8;
+  std::vector<int> us(c->frags.size()), iu(c->frags.size()), ic(c->frags.size());   // storage start; interior units (local)
+  long long tiles = 0;
+  for (size_t f = 0; f < c->frags.size(); ++f) {
+    const DevFrag& F = c->frags[f];
+    if (F.n > 128) {
       t->why = "tensor-core contraction supports at most 128 states per fragment";
       return OFM_OK;
     }
-    ldA = std::max(ldA, A.ld);
-    ldB = std::max(ldB, B.ld);
-    Rb = std::max(Rb, (2 * B.n + 15) / 16 * 16);
+    TcFrag q;
+    unit_range(n0, NU, F.doff[0], F.dext[0], us[f], q.nux);
+    if (q.nux == NU) {   // the whole axis: units outside the box hold zeros
+      iu[f] = 0;
+      ic[f] = NU;
+    } else {
+      int s = 0;
+      unit_range(n0, NU, (F.doff[0] + F.lo[0]) % n0, F.ext[0], s, ic[f]);
+      iu[f] = (s - us[f] + NU) % NU;
+    }
+    q.dext1 = F.dext[1];
+    q.n = F.n;
+    q.rows = (F.n + 7) / 8 * 8;
+    RUnit u;
+    u.frag = (int)f;
+    u.s0[0] = 8 * us[f]; u.s0[1] = F.doff[1]; u.s0[2] = F.doff[2];
+    u.L[0] = 8 * q.nux; u.L[1] = F.dext[1]; u.L[2] = F.dext[2];
+    u.p8 = u.L[0] * u.L[1];
+    u.ntiles = (int)(((long long)u.p8 * u.L[2] + 63) / 64);
+    u.tile0 = tiles;
+    u.base = t->plane_bytes;
+    q.base = u.base;
+    q.npl2 = (long long)u.ntiles * 128 * q.rows;
+    tiles += u.ntiles;
+    t->plane_bytes += (long long)u.ntiles * 64 * q.rows * 8;
+    t->frags.push_back(q);
+    t->units.push_back(u);
+    for (int t0 = 0; t0 < u.ntiles; t0 += 4)
+      t->pack_cta.push_back(make_int4((int)f, t0, std::min(4, u.ntiles - t0), 0));
   }
-  const long long target = chunk > 0 ? chunk : std::max<long long>(1024, kh / (4 * 152));
-  for (size_t p = 0; p < prs.size(); ++p) {
-    const HostPair& hp = prs[p];
-    const DevFrag& B = fr[hp.b];
+  const long long target = c->asm_chunk > 0 ? c->asm_chunk : std::max<long long>(1024, c->kh / (4 * 152));
+  for (size_t p = 0; p < c->pairs.size(); ++p) {
+    const HostPair& hp = c->pairs[p];
+    const DevFrag &A = c->frags[hp.a], &B = c->frags[hp.b];
+    const TcFrag& TB = t->frags[hp.b];
     TcPair tq;
     tq.a = hp.a;
     tq.b = hp.b;
-    tq.N = 2 * B.n;
-    tq.Npad = (tq.N + 15) / 16 * 16;
-    tq.blk_off = blk_off[p];
+    tq.blk_off = c->simt_pairs[p].blk_off;
     tq.item0 = (int)t->items.size();
-    for (const Piece& pc : hp.pieces) {
-      const int pid = (int)t->pieces.size();
-      t->pieces.push_back(pc);
-      const int rows = pc.len[1] * pc.len[2];
-      const int per = (int)std::max<long long>(1, target / pc.len[0]);
-      for (int r0 = 0; r0 < rows; r0 += per) {
-        TcItem it;
-        it.pair = (int)p;
-        it.piece = pid;
-        it.r0 = r0;
-        it.r1 = std::min(rows, r0 + per);
-        it.part_off = t->part_elems;
-        t->part_elems += (long long)fr[hp.a].n * tq.N;
-        t->items.push_back(it);
-      }
-    }
+    // x in units, y and z in points
+    std::vector<Run> runs[3];
+    runs[0] = dim_runs(NU, (us[hp.a] + iu[hp.a]) % NU, ic[hp.a], us[hp.b], TB.nux);
+    for (int d = 1; d < 3; ++d)
+      runs[d] = dim_runs(c->grid.n[d], (A.doff[d] + A.lo[d]) % c->grid.n[d], A.ext[d], B.doff[d], B.dext[d]);
+    long long xpts = 0, xunits = 0;   // shared points per row, and units they take
+    for (const Run& r : dim_runs(n0, (A.doff[0] + A.lo[0]) % n0, A.ext[0], B.doff[0], B.dext[0])) xpts += r.len;
+    for (const Run& r : runs[0]) xunits += r.len;
+    for (const Run& rz : runs[2])
+      for (const Run& ry : runs[1])
+        for (const Run& rx : runs[0]) {
+          const int rows = ry.len * rz.len;
+          // The FP32 accumulation in tensor memory drops bits at every step, so an
+          // item has as many units as its shared points fill (above a minimum): units
+          // padded with zeros must not lengthen the sum.
+          const long long pts = rx.len * xpts * rows / xunits;
+          const long long units = std::max(std::min<long long>(TS_MINUNITS, target / 8), std::min(target, pts) / 8);
+          const int per = (int)std::max<long long>(1, units / rx.len);
+          for (int r0 = 0; r0 < rows; r0 += per) {
+            TcItem it;
+            it.pair = (int)p;
+            it.la[0] = iu[hp.a] + rx.ta; it.la[1] = A.lo[1] + ry.ta; it.la[2] = A.lo[2] + rz.ta;
+            it.lb[0] = rx.lb; it.lb[1] = ry.lb; it.lb[2] = rz.lb;
+            it.m = rx.len;
+            it.leny = ry.len;
+            it.r0 = r0;
+            it.r1 = std::min(rows, r0 + per);
+            it.part_off = t->part_elems;
+            t->part_elems += (long long)A.n * 2 * B.n;
+            t->items.push_back(it);
+          }
+        }
     tq.nitem = (int)t->items.size() - tq.item0;
     t->pairs.push_back(tq);
   }
-  for (int k = 0; k < TC_NKIND; ++k) {
-    SmemLayout& L = t->lay[k];
-    L.ldA = ldA;
-    L.ldB = ldB;
-    L.Rb = Rb;
-    const int esz = (k == TC_TF32 || k == TC_TF32X3) ? 4 : 2;
-    L.ntiles = (k == TC_BF16X3 || k == TC_TF32X3) ? 2 : 1;
-    L.nitems = (int)t->items.size();
-    // the longest K step, then the largest raw stages (fewest per-stage
-    // costs), then the deepest operand ring, that leave two raw stages
-    const long long budget = 216 * 1024;
-    L.nraw = 0;
-    for (L.kt = 64; L.kt >= 32 && L.nraw < 2; L.kt /= 2) {
-      L.tileA = (128 * L.kt * esz + 1023) / 1024 * 1024;
-      L.tileB = (Rb * L.kt * esz + 1023) / 1024 * 1024;
-      for (L.rsteps = 128 / L.kt; L.rsteps >= 1; L.rsteps /= 2) {
-        L.raw_stage = (L.rsteps * L.kt * (ldA + 2 * ldB) * 4 + 1023) / 1024 * 1024;
-        for (L.nop = TS_NOP; L.nop >= 2; --L.nop) {
-          const long long ops = (long long)L.nop * L.ntiles * (L.tileA + L.tileB);
-          L.nraw = (int)std::min<long long>(TS_MAXRAW, (budget - ops) / L.raw_stage);
-          if (L.nraw >= 2) break;
-        }
-        if (L.nraw >= 2) break;
-      }
-      if (L.nraw >= 2) break;
-    }
-    // a kind whose staging does not fit stays unusable (nraw < 2); the others run
-    t->smem[k] = L.nraw >= 2 ? (size_t)L.nraw * L.raw_stage + (size_t)L.nop * L.ntiles * (L.tileA + L.tileB) : 0;
-  }
-  OFM_TRY(ofm_ensure(c, t->d_pairs, sizeof(TcPair) * std::max<size_t>(1, t->pairs.size()), "tc pairs"));
-  OFM_TRY(ofm_ensure(c, t->d_items, sizeof(TcItem) * std::max<size_t>(1, t->items.size()), "tc items"));
-  OFM_TRY(ofm_ensure(c, t->d_pieces, sizeof(Piece) * std::max<size_t>(1, t->pieces.size()), "tc pieces"));
-  OFM_TRY(ofm_ensure(c, t->partials, sizeof(float) * std::max<long long>(1, t->part_elems), "tc partials"));
-  OFM_CUDA(c, cudaMemcpyAsync(t->d_pairs.p, t->pairs.data(), sizeof(TcPair) * t->pairs.size(), cudaMemcpyHostToDevice, c->stream));
-  OFM_CUDA(c, cudaMemcpyAsync(t->d_items.p, t->items.data(), sizeof(TcItem) * t->items.size(), cudaMemcpyHostToDevice, c->stream));
-  OFM_CUDA(c, cudaMemcpyAsync(t->d_pieces.p, t->pieces.data(), sizeof(Piece) * t->pieces.size(), cudaMemcpyHostToDevice, c->stream));
-  static bool attr = false;   // the kernels' shared-memory limit, once per process
-  if (!attr) {
-    set_smem_attr<TC_TF32, 32>();
-    set_smem_attr<TC_BF16, 32>();
-    set_smem_attr<TC_BF16X3, 32>();
-    set_smem_attr<TC_TF32X3, 32>();
-    set_smem_attr<TC_TF32, 64>();
-    set_smem_attr<TC_BF16, 64>();
-    set_smem_attr<TC_BF16X3, 64>();
-    set_smem_attr<TC_TF32X3, 64>();
-    OFM_CUDA(c, cudaGetLastError());
-    attr = true;
-  }
+  t->order.resize(t->items.size());
+  for (size_t i = 0; i < t->order.size(); ++i) t->order[i] = (int)i;
+  auto cost = [&](int i) {
+    const TcItem& it = t->items[i];
+    const TcPair& q = t->pairs[it.pair];
+    return (long long)(it.r1 - it.r0) * it.m * (t->frags[q.a].rows + 2 * t->frags[q.b].rows);
+  };
+  std::stable_sort(t->order.begin(), t->order.end(), [&](int x, int y) { return cost(x) > cost(y); });
   t->ok = true;
   return OFM_OK;
 }
 
-// Plan of the pair contraction after a build.
-ofm_status ofm_plan_extra(ofm_ctx* c) {
-  if (c->storage != OFM_STORE_FP32) {
-    if (!c->tc) c->tc = new TcPlan();
-    c->tc->ok = false;
-    c->tc->why = "tensor-core contraction needs FP32 storage";
-    return OFM_OK;
-  }
-  std::vector<long long> off(c->pairs.size());
-  for (size_t p = 0; p < c->pairs.size(); ++p) off[p] = c->simt_pairs[p].blk_off;
-  return ofm_tc_plan_build(c, &c->tc, c->frags, c->pairs, off, c->kh, c->asm_chunk);
+template <typename T>
+static ofm_status put(ofm_ctx* c, DevBuf& b, const std::vector<T>& v, const char* what) {
+  OFM_TRY(ofm_ensure(c, b, sizeof(T) * std::max<size_t>(1, v.size()), what));
+  if (!v.empty()) OFM_CUDA(c, cudaMemcpyAsync(b.p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, c->stream));
+  return OFM_OK;
 }
 
-template <int KIND>
-static void launch_kind(const TcPlan* t, int kt, int grid, size_t sm, cudaStream_t s,
-                        const DevFrag* fr, const float* st, const float* hp, int* fl) {
-  const SmemLayout& L = t->lay[KIND];
-  const TcPair* pr = (const TcPair*)t->d_pairs.p;
-  const Piece* pc = (const Piece*)t->d_pieces.p;
-  const TcItem* itm = (const TcItem*)t->d_items.p;
-  float* part = (float*)t->partials.p;
-  if (kt == 64)
-    tc_contract_kernel<KIND, 64><<<grid, TS_THREADS, sm, s>>>(fr, pr, pc, itm, st, hp, part, fl, L);
-  else
-    tc_contract_kernel<KIND, 32><<<grid, TS_THREADS, sm, s>>>(fr, pr, pc, itm, st, hp, part, fl, L);
-}
-
-// Runs a plan: contraction into FP32 partials, then the fixed-order sum into
-// the FP64 block arena.  kind: TC_TF32 .. TC_TF32X3.
-ofm_status ofm_tc_run(ofm_ctx* c, TcPlan* t, int kind, const DevFrag* d_frags, const void* states,
-                      const void* hphi, double* blocks, int kclass_contract, int kclass_finalize,
-                      double bytes, double flops) {
+// Device tables (after a re-plan) and buffers, made before any capture.
+ofm_status ofm_tc_prepare(ofm_ctx* c, ofm_precision prec) {
+  (void)prec;
+  TcPlan* t = c->tc;
   if (!t || !t->ok) return ofm_fail(c, OFM_ERR_INVALID, t ? t->why : "no tensor-core plan");
-  if (!ofm_tc_plan_ok(t, kind))
-    return ofm_fail(c, OFM_ERR_INVALID, "tensor-core staging does not fit shared memory for these state counts");
-  const int nit = (int)t->items.size();
+  void* arena = nullptr;
+  OFM_TRY(ofm_pair_planes(c, std::max<long long>(16, t->plane_bytes), &arena));
+  OFM_TRY(ofm_ensure_big(c, t->partials, sizeof(float) * (size_t)std::max<long long>(1, t->part_elems), "tc partials"));
+  if (t->uploaded) return OFM_OK;
+  OFM_TRY(put(c, t->d_frags, t->frags, "tc fragments"));
+  OFM_TRY(put(c, t->d_units, t->units, "tc pack units"));
+  OFM_TRY(put(c, t->d_pcta, t->pack_cta, "tc pack table"));
+  OFM_TRY(put(c, t->d_pairs, t->pairs, "tc pairs"));
+  OFM_TRY(put(c, t->d_items, t->items, "tc items"));
+  OFM_TRY(put(c, t->d_order, t->order, "tc item order"));
+  static bool attr = false;   // the kernels' shared-memory limit, once per process
+  if (!attr) {
+    cudaFuncSetAttribute(tc_contract_kernel<TC_TF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM);
+    cudaFuncSetAttribute(tc_contract_kernel<TC_BF16>, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM);
+    cudaFuncSetAttribute(tc_contract_kernel<TC_BF16X3>, cudaFuncAttributeMaxDynamicSharedMemorySize, TS_SMEM);
+    OFM_CUDA(c, cudaGetLastError());
+    attr = true;
+  }
+  t->uploaded = true;
+  return OFM_OK;
+}
+
+// a1 (H phi and the operand planes), a3/a4 (contraction into FP32 partials) and
+// a5 (the fixed-order sum into the FP64 block arena) on the context stream.
+ofm_status ofm_contract_tc(ofm_ctx* c, ofm_precision prec) {
+  TcPlan* t = c->tc;
+  if (!t || !t->ok) return ofm_fail(c, OFM_ERR_INVALID, t ? t->why : "no tensor-core plan");
+  if (!t->uploaded) return ofm_fail(c, OFM_ERR_STATE, "tensor-core plan not prepared");
+  const int kind = prec == OFM_PREC_TF32 ? TC_TF32 : prec == OFM_PREC_BF16 ? TC_BF16 : TC_BF16X3;
+  void* arena = nullptr;
+  OFM_TRY(ofm_pair_planes(c, std::max<long long>(16, t->plane_bytes), &arena));
+  OFM_TRY(ofm_pair_pack(c, kind, (const RUnit*)t->d_units.p, (const int4*)t->d_pcta.p, (int)t->pack_cta.size(), arena,
+                        t->plane_bytes));
   int* fl = (int*)c->flag.p + OFM_FLAG_TC;
+  int* next = (int*)c->flag.p + OFM_FLAG_QUEUE;
+  OFM_CUDA(c, cudaMemsetAsync(next, 0, sizeof(int), c->stream));
+  const TcFrag* fr = (const TcFrag*)t->d_frags.p;
+  const TcPair* pr = (const TcPair*)t->d_pairs.p;
+  const TcItem* it = (const TcItem*)t->d_items.p;
   {
-    KTimer kt(c, kclass_contract, 1, bytes, flops);
-    if (nit > 0) {
-      const int grid = std::min(nit, 152);   // one persistent CTA per SM
-      const int ktl = t->lay[kind].kt;
-      const size_t sm = t->smem[kind];
-      const float* st = (const float*)states;
-      const float* hp = (const float*)hphi;
-      if (kind == TC_TF32) launch_kind<TC_TF32>(t, ktl, grid, sm, c->stream, d_frags, st, hp, fl);
-      else if (kind == TC_BF16) launch_kind<TC_BF16>(t, ktl, grid, sm, c->stream, d_frags, st, hp, fl);
-      else if (kind == TC_BF16X3) launch_kind<TC_BF16X3>(t, ktl, grid, sm, c->stream, d_frags, st, hp, fl);
-      else launch_kind<TC_TF32X3>(t, ktl, grid, sm, c->stream, d_frags, st, hp, fl);
+    KTimer kt(c, KC_CONTRACT, 1, c->contract_bytes, (double)c->flops);
+    const int ni = (int)t->items.size(), grid = std::min(ni, 152);   // one persistent CTA per SM
+    const int* od = (const int*)t->d_order.p;
+    const unsigned char* pl = (const unsigned char*)arena;
+    float* pa = (float*)t->partials.p;
+    if (ni > 0) {
+      if (kind == TC_TF32) tc_contract_kernel<TC_TF32><<<grid, TS_THREADS, TS_SMEM, c->stream>>>(fr, pr, it, od, ni, pl, pa, fl, next);
+      else if (kind == TC_BF16) tc_contract_kernel<TC_BF16><<<grid, TS_THREADS, TS_SMEM, c->stream>>>(fr, pr, it, od, ni, pl, pa, fl, next);
+      else tc_contract_kernel<TC_BF16X3><<<grid, TS_THREADS, TS_SMEM, c->stream>>>(fr, pr, it, od, ni, pl, pa, fl, next);
     }
     OFM_CUDA(c, cudaGetLastError());
   }
   {
-    KTimer kt(c, kclass_finalize, 1, (double)t->part_elems * 4);
-    // enough output chunks for the largest block (n_a <= 128, n_b = N / 2)
-    int nmax = 1;
-    for (const TcPair& q : t->pairs) nmax = std::max(nmax, q.N / 2);
-    const int chunks = std::max(1, (128 * nmax + 255) / 256);
+    KTimer kt(c, KC_FINALIZE, 1, (double)t->part_elems * 4);
+    int amax = 1, bmax = 1;
+    for (const TcPair& q : t->pairs) {
+      amax = std::max(amax, t->frags[q.a].n);
+      bmax = std::max(bmax, t->frags[q.b].n);
+    }
     if (!t->pairs.empty())
-      tc_finalize_kernel<<<dim3((int)t->pairs.size(), chunks), 256, 0, c->stream>>>(
-          d_frags, (const TcPair*)t->d_pairs.p, (const TcItem*)t->d_items.p,
-          (const float*)t->partials.p, blocks);
+      tc_finalize_kernel<<<dim3((int)t->pairs.size(), (amax * bmax + 255) / 256), 256, 0, c->stream>>>(
+          fr, pr, it, (const float*)t->partials.p, (double*)c->blocks.p);
     OFM_CUDA(c, cudaGetLastError());
   }
   c->tc_check = true;
   return OFM_OK;
-}
-
-ofm_status ofm_contract_tc(ofm_ctx* c, ofm_precision prec) {
-  const int kind = prec == OFM_PREC_TF32 ? TC_TF32 : prec == OFM_PREC_BF16 ? TC_BF16 : TC_BF16X3;
-  return ofm_tc_run(c, c->tc, kind, (const DevFrag*)c->d_frags.p, c->states.p, c->hphi.p,
-                    (double*)c->blocks.p, KC_CONTRACT, KC_FINALIZE, c->contract_bytes, (double)c->flops);
 }
 
 // Reports a bounded-wait timeout of an earlier tensor-core or staged-stencil
