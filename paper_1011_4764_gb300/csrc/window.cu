@@ -1,9 +1,9 @@
 // FP64 solution of the generalized eigenproblem of Eq. 2,
 //     sum_mn (H - E S) C = 0,
 // for the eigenvalues inside an energy window, on the device:
-//   1. Cholesky S = L L^T (blocked, right-looking, 32-wide panels);
-//   2. A = L^-1 H L^-T by two blocked forward substitutions with the
-//      block multipliers L_jj^-1 and L_ij L_jj^-1 formed once;
+//   1. Cholesky S = L L^T (blocked, right-looking, 32-wide panels with inverted
+//      diagonal blocks) and, in the same sweep, X = L^-1 H;
+//   2. A = L^-1 X^T, on and above the diagonal;
 //   3. Householder reduction of A to a symmetric tridiagonal T (d, e);
 //   4. Sturm-sequence counts and bisection on T, one thread per wanted
 //      eigenvalue index.
@@ -17,206 +17,359 @@
 #include <cmath>
 #include <vector>
 
+#include "fp64_util.h"
 #include "ofm_internal.h"
 
 namespace ofm {
 
 constexpr int NB = 32;
 
-// ---------------------------------------------------------------- Cholesky --
+// ------------------------------------------ Cholesky and reduction to A ------
+//
+// In blocks of NB rows.  With Q_j = L_jj^-1, block column j of the factor and
+// block row j of X = L^-1 H come from the same two launches:
+//   panel:  L_ij = S_ij Q_j^T (i > j),        X_j = Q_j H_j;
+//   update: S_ik -= L_ij L_kj^T (i >= k > j), H_i -= L_ij X_j (i > j),
+// and the CTA that updates the next diagonal block goes on to factor and invert
+// it while the other CTAs work on the rest of the update.  The second half,
+// A = L^-1 X^T, forms only the blocks on and above the diagonal (A_jc, c >= j,
+// needs A_kc with k < j <= c only) and mirrors them: a third of the work of the
+// full solve, one launch per block row, whose CTAs on row j + 1 multiply by
+// Q_{j+1} right after their update.
+//
+// FP64 issue bounds all of it (one warp instruction per 17 cycles and SM), so an
+// item is a 32 x 16 strip, 512 of them (4.3 us), handed out by a counter to one
+// CTA per SM, the next item's operands on their way while one is computed; one
+// CTA per SM keeps the pipe of the factoring CTA free of other CTAs' work.
+// n = 992: 1.95 (Cholesky) + 2.42 ms with substitutions, separate sweeps and
+// the full second solve; 1.89 (factor and X) + 0.68 now.  n = 315: 0.58 + 0.35 ms;
+// 0.36 + 0.14 now.
 
-// Factor the kb x kb diagonal block at (k0, k0) in place (lower triangle).
-// Column j of the working copy stays unscaled; its pivot's reciprocal square
-// root r_j and r_j^2 are formed by ONE thread (an FP64 square root and a
-// division are long instruction sequences on a part with few FP64 units):
-// the thread that applies column j's update to the next pivot forms the
-// next r right away, while the other rows finish their updates, so each
-// column costs one barrier and no serial scalar step of its own.  The
-// update is a_yx -= a_yj (a_xj r_j^2); the scaling L_yj = a_yj r_j is applied
-// on the way out (L_jj = piv r_j).
-__global__ void potrf_diag_kernel(double* W, int n, int k0, int kb, int* fail_col) {
-  __shared__ double a[NB][NB + 1];
-  __shared__ double rinv[NB], r2[NB];
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 32
-  if (tx < kb && ty < kb) a[ty][tx] = W[(long long)(k0 + ty) * n + k0 + tx];
-  __syncthreads();
-  // r of the pivot at (j, j), which no later update of this block touches
-  auto pivot = [&](int j) {
-    double piv = a[j][j];
-    if (!(piv > 0.0)) {
-      atomicCAS(fail_col, -1, k0 + j);
-      piv = 1.0;  // keep going with finite numbers; the call reports failure
-      a[j][j] = 1.0;
-    }
-    const double r = rsqrt(piv);
-    rinv[j] = r;
-    r2[j] = r * r;
+constexpr int ST_C = 16;               // columns of a strip
+constexpr int ST_THREADS = 256;
+constexpr size_t ST_SMEM = 120 * 1024; // more than half an SM's shared memory: one CTA per SM
+
+struct StepSmem {
+  double li[2][NB][NB + 1];   // L_ij of the item, double-buffered
+  double b[2][NB][ST_C + 1];  // the strip of L_kj^T, X_j or A_j
+  double q[NB][NB + 1];       // Q of the next diagonal block, or the block being factored
+  double t[NB][NB + 1];       // a strip on its way through Q; unscaled columns of L
+  double g[2][NB], h[2][NB], piv[NB];
+  int item;
+};
+static_assert(sizeof(StepSmem) <= ST_SMEM, "strip buffers fit");
+
+// Eight bytes into shared memory, asynchronously; zeros where !ok.
+__device__ __forceinline__ void cpa8z(double* dst, const double* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+               "l"((unsigned long long)__cvta_generic_to_global(src)), "r"(ok ? 8 : 0)
+               : "memory");
+}
+
+__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cpa_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// 32 x 32 block at (r0, k0) of an n x n matrix into d.
+__device__ __forceinline__ void fetch_block(double (*d)[NB + 1], const double* M, int n, int r0, int k0) {
+  for (int e = threadIdx.x; e < NB * NB; e += ST_THREADS) {
+    const int r = e >> 5, c = e & 31;
+    const bool ok = r0 + r < n && k0 + c < n;
+    cpa8z(&d[r][c], ok ? M + (size_t)(r0 + r) * n + k0 + c : M, ok);
+  }
+}
+// strip d[t][c] = M(k0 + t, c0 + c), or M(c0 + c, k0 + t) when transposed
+template <bool TR>
+__device__ __forceinline__ void fetch_strip(double (*d)[ST_C + 1], const double* M, int n, int k0, int c0) {
+  for (int e = threadIdx.x; e < NB * ST_C; e += ST_THREADS) {
+    const int t = TR ? e & 31 : e >> 4, c = TR ? e >> 5 : e & 15;
+    const bool ok = k0 + t < n && c0 + c < n;
+    cpa8z(&d[t][c], ok ? (TR ? M + (size_t)(c0 + c) * n + k0 + t : M + (size_t)(k0 + t) * n + c0 + c) : M, ok);
+  }
+}
+
+// Factor the symmetric block a (identity beyond kb) as L L^T and invert L, in
+// one elimination without square roots: row y > j takes -(a_yj / d_j) times row
+// j, whose entries left of j hold the inverse of the unit factor so far; the
+// scaling by d^-1/2 follows for all columns at once.  A column costs one barrier
+// and the chain update - reciprocal - scaling of the next pivot row, which warp 0
+// works on with an FP64 sub-partition to itself (warp 4, its neighbour there, only
+// waits).  The six warps on the others own the rows and hand row j + 2 over while
+// warp 0 works on row j + 1.  Eight warps taking turns as the next pivot's
+// owner, each step waiting for its neighbour's updates: 27 us a block; now 23.
+__device__ void factor_block(StepSmem& sm, double (*a)[NB + 1], int kb, double* W, double* Qj, int n, int k0,
+                             int* fail_col) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int own = warp == 0 || warp == 4 ? -1 : warp - (warp > 4 ? 2 : 1);   // 0..5: rows own, own + 6, ..
+  double v[6];
+  if (own >= 0)
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v[q] = own + 6 * q < NB ? a[own + 6 * q][lane] : 0.0;
+  // row y: subtract a_yj times the published row; column j turns into the inverse's
+  auto update = [&](double row, double gx, int y, int j) {
+    const double ay = __shfl_sync(0xffffffffu, row, j);
+    if (lane == j) sm.t[y][j] = ay;
+    return fma(-ay, gx, lane == j ? 0.0 : row);
   };
-  if (tx == 0 && ty == 0) pivot(0);
+  auto publish = [&](double row, int j) {   // row j, all updates in
+    double p = __shfl_sync(0xffffffffu, row, j);
+    if (!(p > 0.0)) {
+      if (lane == 0) atomicCAS(fail_col, -1, k0 + j);
+      p = 1.0;   // keep going with finite numbers; the call reports failure
+    }
+    const double r = rcp64(p);
+    sm.g[j & 1][lane] = lane == j ? r : row * r;
+    if (lane == j) sm.piv[j] = p;
+    a[j][lane] = row;
+  };
+  __syncthreads();   // the rows are in registers; a takes the finished ones
+  if (warp == 0) publish(a[0][lane], 0);
+  if (own == 1) sm.h[0][lane] = v[0];   // row 1 before any update
   __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (ty > j && ty < kb && tx > j && tx <= ty) {
-      a[ty][tx] = fma(-a[ty][j], a[tx][j] * r2[j], a[ty][tx]);
-      if (tx == j + 1 && ty == j + 1) pivot(j + 1);
+  for (int j = 0; j + 1 < NB; ++j) {
+    const double gx = sm.g[j & 1][lane];
+    if (warp == 0) {
+      publish(update(sm.h[j & 1][lane], gx, j + 1, j), j + 1);
+    } else if (own >= 0) {
+      const int y2 = j + 2;
+#pragma unroll
+      for (int q = 0; q < 6; ++q)
+        if (own + 6 * q == y2 && y2 < NB) {
+          v[q] = update(v[q], gx, y2, j);
+          sm.h[(j + 1) & 1][lane] = v[q];
+        }
+#pragma unroll
+      for (int q = 0; q < 6; ++q)
+        if (own + 6 * q > y2 && own + 6 * q < NB) v[q] = update(v[q], gx, own + 6 * q, j);
     }
     __syncthreads();
   }
-  if (tx < kb && ty < kb && tx <= ty) W[(long long)(k0 + ty) * n + k0 + tx] = a[ty][tx] * rinv[tx];
-}
-
-// Rows i >= k0+kb of the panel: L21 = W21 L11^-T (forward substitution per
-// row).  Four lanes share a row (lane = 4 row + phase), each summing every
-// fourth term of x_j = (w_j - sum_{t<j} x_t L_jt) / L_jj, combined by two
-// shuffle levels: one warp issues an FP64 instruction every 64 cycles at
-// best, so a row's ~kb^2/2 products are split four ways rather than chained
-// in one lane.  8 rows per warp, 4 warps per CTA.
-__global__ void __launch_bounds__(128) trsm_panel_kernel(double* W, int n, int k0, int kb) {
-  __shared__ double l[NB][NB + 1];
-  __shared__ double dinv[NB];
-  __shared__ double xs[32][NB + 1];   // solved entries of the CTA's 32 rows
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    int r = e / NB, cc = e % NB;
-    l[r][cc] = (r < kb && cc <= r) ? W[(long long)(k0 + r) * n + k0 + cc] : 0.0;
-  }
-  __syncthreads();
-  for (int j = threadIdx.x; j < kb; j += blockDim.x) dinv[j] = 1.0 / l[j][j];
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rl = warp * 8 + (lane >> 2), ph = lane & 3;   // row within the CTA, phase
-  const int i = k0 + kb + blockIdx.x * 32 + rl;
-  const bool live = i < n;
-  double* row = W + (long long)(live ? i : k0) * n + k0;
-  double* x = xs[rl];
-  for (int j = 0; j < kb; ++j) {
-    double s = 0.0;
-    for (int t = ph; t < j; t += 4) s = fma(x[t], l[j][t], s);
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if (ph == 0) x[j] = live ? (row[j] - s) * dinv[j] : 0.0;
-    __syncwarp();
-  }
-  if (live)
-    for (int j = ph; j < kb; j += 4) row[j] = x[j];
-}
-
-// Trailing update of the lower triangle: W22 -= L21 L21^T (32x32 tiles).
-__global__ void syrk_update_kernel(double* W, int n, int k0, int kb) {
-  const int t0 = k0 + kb;
-  const int bi = blockIdx.y, bj = blockIdx.x;
-  if (bj > bi) return;
-  __shared__ double li[NB][NB + 1], lj[NB][NB + 1];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i0 = t0 + bi * NB, j0 = t0 + bj * NB;
-  {
-    int r = i0 + ty;
-    li[ty][tx] = (r < n && tx < kb) ? W[(long long)r * n + k0 + tx] : 0.0;
-    r = j0 + ty;
-    lj[ty][tx] = (r < n && tx < kb) ? W[(long long)r * n + k0 + tx] : 0.0;
-  }
-  __syncthreads();
-  const int i = i0 + ty, j = j0 + tx;
-  if (i < n && j < n && j <= i) {
-    double s = 0.0;
-#pragma unroll 8
-    for (int t = 0; t < NB; ++t) s += li[ty][t] * lj[tx][t];
-    W[(long long)i * n + j] -= s;
-  }
-}
-
-// ------------------------------------------------------ triangular solves --
-//
-// L X = B is solved by blocks of NB rows with precomputed multipliers
-// Q_jj = L_jj^-1 (diagonal blocks) and Q_ij = L_ij L_jj^-1 (i > j): step j
-// writes X_j = Q_jj B_j and updates B_i -= Q_ij B_j (= L_ij X_j) for i > j,
-// one independent NB x NB x NB product per CTA.  The serial substitutions are
-// confined to the NB x NB diagonal inverses, computed once per factorisation
-// for all blocks in one launch.
-
-// Q_jj = L_jj^-1: one CTA of NB threads per diagonal block, thread c solves
-// L_jj x = e_c by forward substitution (reciprocal pivots); the strictly
-// upper part of the block is written as zero.
-__global__ void inv_diag_kernel(const double* L, double* Q, int n) {
-  __shared__ double l[NB][NB + 1];
-  __shared__ double dinv[NB];
-  const int k0 = blockIdx.x * NB, kb = min(NB, n - k0);
-  const int c = threadIdx.x;
-  for (int r = 0; r < NB; ++r) l[r][c] = (r < kb && c <= r) ? L[(long long)(k0 + r) * n + k0 + c] : 0.0;
-  __syncthreads();
-  if (c < kb) dinv[c] = 1.0 / l[c][c];
-  __syncthreads();
-  if (c >= kb) return;
-  double x[NB];
+  const double d = sm.piv[lane], rs = rsqrt64(d);
 #pragma unroll
-  for (int r = 0; r < NB; ++r) {
-    double v = 0.0;
-    if (r == c) {
-      v = dinv[c];
-    } else if (r > c && r < kb) {
-      double s = 0.0;
-      for (int k = c; k < r; ++k) s -= l[r][k] * x[k];
-      v = s * dinv[r];
+  for (int q = 0; q < 4; ++q) {
+    const int y = warp + 8 * q;
+    const double ry = __shfl_sync(0xffffffffu, rs, y);
+    Qj[y * NB + lane] = lane < y ? a[y][lane] * ry : lane == y ? ry : 0.0;
+    if (y < kb && lane <= y)
+      W[(size_t)(k0 + y) * n + k0 + lane] = lane < y ? sm.t[y][lane] * rs : d * rs;
+  }
+}
+
+// acc of rows row and row + 16 (both at column col): sum over t of l[.][t] b[t][col]
+__device__ __forceinline__ void strip_product(const double (*l)[NB + 1], const double (*b)[ST_C + 1], int row,
+                                              int col, double& a0, double& a1) {
+  a0 = a1 = 0.0;
+#pragma unroll 8
+  for (int t = 0; t < NB; ++t) {
+    const double x = b[t][col];
+    a0 = fma(l[row][t], x, a0);
+    a1 = fma(l[row + 16][t], x, a1);
+  }
+}
+
+// Panel of block j: strips of eight rows of S_ij, then strips of eight columns
+// of H_j, each multiplied by Q_j (lower triangular) in place.
+__global__ void __launch_bounds__(128) panel_kernel(double* W, double* B, const double* __restrict__ Q, int n,
+                                                    int j) {
+  __shared__ double q[NB][NB + 1], b[NB][9];
+  const int k0 = j * NB, below = n - k0 - NB, nl = below > 0 ? (below + 7) / 8 : 0;
+  const bool isl = (int)blockIdx.x < nl;
+  const int x0 = isl ? k0 + NB + 8 * blockIdx.x : 8 * (blockIdx.x - nl);
+  for (int e = threadIdx.x; e < NB * NB; e += 128) q[e >> 5][e & 31] = Q[(size_t)j * NB * NB + e];
+  for (int e = threadIdx.x; e < NB * 8; e += 128) {
+    const int t = isl ? e & 31 : e >> 3, c = isl ? e >> 5 : e & 7;
+    const bool ok = k0 + t < n && x0 + c < n;
+    b[t][c] = !ok ? 0.0 : isl ? W[(size_t)(x0 + c) * n + k0 + t] : B[(size_t)(k0 + t) * n + x0 + c];
+  }
+  __syncthreads();
+  const int col = threadIdx.x & 7, row = threadIdx.x >> 3;
+  double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+  for (int t = 0; t < 16; ++t) {
+    a0 = fma(q[row][t], b[t][col], a0);
+    a1 = fma(q[row + 16][t], b[t][col], a1);
+  }
+#pragma unroll
+  for (int t = 16; t < NB; ++t) a1 = fma(q[row + 16][t], b[t][col], a1);
+  if (x0 + col >= n) return;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int r = k0 + row + 16 * u;
+    if (r >= n) continue;
+    const double v = u ? a1 : a0;
+    if (isl) W[(size_t)(x0 + col) * n + r] = v;
+    else B[(size_t)r * n + x0 + col] = v;
+  }
+}
+
+// Takes the CTA's next item (a uniform value; -1 when none is left).
+__device__ __forceinline__ int claim(StepSmem& sm, int* next, int total) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const int t = atomicAdd(next, 1);
+    sm.item = t < total ? t : -1;
+  }
+  __syncthreads();
+  return sm.item;
+}
+
+// Update after panel j; CTA 0 first updates, factors and inverts block j + 1
+// (j = -1: factors block 0, with nothing to update).
+__global__ void __launch_bounds__(ST_THREADS) factor_step_kernel(double* W, double* B, double* Q, int n, int j,
+                                                                 int* next, int* fail_col) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  StepSmem& sm = *reinterpret_cast<StepSmem*>(raw);
+  const int nblk = (n + NB - 1) / NB, nstr = (n + ST_C - 1) / ST_C;
+  const int R = nblk - 1 - j, k0 = j * NB, i0 = k0 + NB;
+  const int tid = threadIdx.x, col = tid & 15, row = tid >> 4;
+  if (blockIdx.x == 0) {
+    const int kb = min(NB, n - i0);
+    if (j >= 0) fetch_block(sm.li[0], W, n, i0, k0);
+    cpa_commit();
+    cpa_wait<0>();
+    __syncthreads();
+    for (int e = tid; e < NB * NB; e += ST_THREADS) {
+      const int r = e >> 5, c = e & 31;
+      double v = r == c ? 1.0 : 0.0;
+      if (r < kb && c < kb) {
+        v = W[(size_t)(i0 + max(r, c)) * n + i0 + min(r, c)];
+        if (j >= 0) {
+          double s = 0.0;
+#pragma unroll 8
+          for (int t = 0; t < NB; ++t) s = fma(sm.li[0][r][t], sm.li[0][c][t], s);
+          v -= s;
+        }
+      }
+      sm.q[r][c] = v;
     }
-    x[r] = v;
+    __syncthreads();
+    factor_block(sm, sm.q, kb, W, Q + (size_t)(j + 1) * NB * NB, n, i0, fail_col);
   }
-#pragma unroll
-  for (int r = 0; r < NB; ++r)
-    if (r < kb) Q[(long long)(k0 + r) * n + k0 + c] = x[r];
+  if (j < 0) return;
+  // items: strips of the lower blocks of S but the two of block j + 1, then all of H
+  const int ns = R * (R + 1) - 2, total = ns + R * nstr;
+  auto place = [&](int t, int& r0, int& c0) {   // returns whether the item is one of S
+    if (t < ns) {
+      int r = (int)((sqrtf(4.f * (t + 2) + 1.f) - 1.f) * 0.5f);   // r (r + 1) <= t + 2
+      while ((r + 1) * (r + 2) <= t + 2) ++r;
+      while (r * (r + 1) > t + 2) --r;
+      r0 = i0 + NB * r;
+      c0 = i0 + ST_C * (t + 2 - r * (r + 1));
+      return true;
+    }
+    const int r = (t - ns) / nstr;
+    r0 = i0 + NB * r;
+    c0 = ST_C * (t - ns - r * nstr);
+    return false;
+  };
+  auto fetch = [&](int t, int buf) {
+    if (t >= 0) {
+      int r0, c0;
+      const bool s = place(t, r0, c0);
+      fetch_block(sm.li[buf], W, n, r0, k0);
+      if (s) fetch_strip<true>(sm.b[buf], W, n, k0, c0);
+      else fetch_strip<false>(sm.b[buf], B, n, k0, c0);
+    }
+    cpa_commit();
+  };
+  int cur = claim(sm, next, total), buf = 0;
+  fetch(cur, 0);
+  while (cur >= 0) {
+    const int nxt = claim(sm, next, total);
+    fetch(nxt, buf ^ 1);
+    cpa_wait<1>();
+    __syncthreads();
+    int r0, c0;
+    double* M = place(cur, r0, c0) ? W : B;
+    double* o0 = M + (size_t)(r0 + row) * n + c0 + col;
+    double* o1 = o0 + (size_t)16 * n;
+    const bool w0 = c0 + col < n && r0 + row < n, w1 = c0 + col < n && r0 + row + 16 < n;
+    const double p0 = w0 ? *o0 : 0.0, p1 = w1 ? *o1 : 0.0;
+    double a0, a1;
+    strip_product(sm.li[buf], sm.b[buf], row, col, a0, a1);
+    if (w0) *o0 = p0 - a0;
+    if (w1) *o1 = p1 - a1;
+    cur = nxt;
+    buf ^= 1;
+  }
+  cpa_wait<0>();
 }
 
-// Q_ij = L_ij Q_jj for the blocks below the diagonal (grid: j, i).
-__global__ void panel_mul_kernel(const double* L, double* Q, int n) {
-  const int j = blockIdx.x, i = blockIdx.y;
-  if (i <= j) return;
-  __shared__ double a[NB][NB + 1], q[NB][NB + 1];
-  const int r0 = i * NB, k0 = j * NB;
-  const int rb = min(NB, n - r0), kb = min(NB, n - k0);
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, cc = e % NB;
-    a[r][cc] = (r < rb && cc < kb) ? L[(long long)(r0 + r) * n + k0 + cc] : 0.0;
-    q[r][cc] = (r < kb && cc < kb) ? Q[(long long)(k0 + r) * n + k0 + cc] : 0.0;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, cc = e % NB;
-    double s = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < NB; ++k) s = fma(a[r][k], q[k][cc], s);
-    if (r < rb && cc < kb) Q[(long long)(r0 + r) * n + k0 + cc] = s;
-  }
-}
-
-// Step j: block row i = j + blockIdx.y, columns c0 = NB blockIdx.x ..
-//   i == j: X_j = Q_jj B_j;   i > j: B_i -= Q_ij B_j.
-__global__ void __launch_bounds__(256) trsm_step_kernel(const double* Q, double* B, double* X,
-                                                        int n, int j) {
-  __shared__ double q[NB][NB + 1], bj[NB][NB + 1];
-  const int i = j + blockIdx.y, c0 = blockIdx.x * NB;
-  const int r0 = i * NB, k0 = j * NB;
-  const int rb = min(NB, n - r0), kb = min(NB, n - k0), cb = min(NB, n - c0);
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, cc = e % NB;
-    q[r][cc] = (r < rb && cc < kb) ? Q[(long long)(r0 + r) * n + k0 + cc] : 0.0;
-    bj[r][cc] = (r < kb && cc < cb) ? B[(long long)(k0 + r) * n + c0 + cc] : 0.0;
-  }
-  __syncthreads();
-  // four outputs per thread: rows ty, ty + 8, ty + 16, ty + 24 of column tx
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 8
-  for (int k = 0; k < NB; ++k) {
-    const double b = bj[k][tx];
+// Second half after block row j of A: T_i -= L_ij A_j on and right of the
+// diagonal, and A_{j+1} = Q_{j+1} T_{j+1}, written to both triangles of A
+// (j = -1: only A_0 = Q_0 T_0).
+__global__ void __launch_bounds__(ST_THREADS) reduce_step_kernel(const double* __restrict__ L,
+                                                                 const double* __restrict__ Q, double* T,
+                                                                 double* A, int n, int j, int* next) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  StepSmem& sm = *reinterpret_cast<StepSmem*>(raw);
+  const int nblk = (n + NB - 1) / NB, nstr = (n + ST_C - 1) / ST_C;
+  const int k0 = j * NB, i0 = k0 + NB;
+  const int R = j < 0 ? 1 : nblk - 1 - j;      // block rows to update
+  const int S0 = nstr - 2 * (j + 1);           // strips of the first; two fewer on each next
+  const int tid = threadIdx.x, col = tid & 15, row = tid >> 4;
+  const int total = R * S0 - R * (R - 1);
+  for (int e = tid; e < NB * NB; e += ST_THREADS) sm.q[e >> 5][e & 31] = Q[(size_t)(j + 1) * NB * NB + e];
+  auto place = [&](int t, int& r0, int& c0) {   // r: r S0 - r (r - 1) <= t
+    const float h = 0.5f * (S0 + 1);
+    int r = (int)(h - sqrtf(fmaxf(h * h - (float)t, 0.f)));
+    r = max(0, min(r, R - 1));
+    while (r + 1 < R && (r + 1) * S0 - (r + 1) * r <= t) ++r;
+    while (r > 0 && r * S0 - r * (r - 1) > t) --r;
+    r0 = i0 + NB * r;
+    c0 = r0 + ST_C * (t - (r * S0 - r * (r - 1)));
+  };
+  auto fetch = [&](int t, int buf) {
+    if (t >= 0 && j >= 0) {
+      int r0, c0;
+      place(t, r0, c0);
+      fetch_block(sm.li[buf], L, n, r0, k0);
+      fetch_strip<false>(sm.b[buf], A, n, k0, c0);
+    }
+    cpa_commit();
+  };
+  int cur = claim(sm, next, total), buf = 0;
+  fetch(cur, 0);
+  while (cur >= 0) {
+    const int nxt = claim(sm, next, total);
+    fetch(nxt, buf ^ 1);
+    cpa_wait<1>();
+    __syncthreads();
+    int r0, c0;
+    place(cur, r0, c0);
+    double* o0 = T + (size_t)(r0 + row) * n + c0 + col;
+    double* o1 = o0 + (size_t)16 * n;
+    const bool w0 = c0 + col < n && r0 + row < n, w1 = c0 + col < n && r0 + row + 16 < n;
+    const double p0 = w0 ? *o0 : 0.0, p1 = w1 ? *o1 : 0.0;
+    double a0 = 0.0, a1 = 0.0;
+    if (j >= 0) strip_product(sm.li[buf], sm.b[buf], row, col, a0, a1);
+    a0 = p0 - a0;
+    a1 = p1 - a1;
+    if (r0 == i0) {
+      __syncthreads();   // the strip of A_j is read
+      sm.b[buf][row][col] = a0;
+      sm.b[buf][row + 16][col] = a1;
+      __syncthreads();
+      strip_product(sm.q, sm.b[buf], row, col, a0, a1);
+      const int c = c0 + col;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = fma(q[ty + 8 * u][k], b, acc[u]);
+      for (int u = 0; u < 2; ++u) {
+        const int r = r0 + row + 16 * u;
+        if (r < n && c < n && c >= r) {
+          A[(size_t)r * n + c] = u ? a1 : a0;
+          A[(size_t)c * n + r] = u ? a1 : a0;
+        }
+      }
+    } else {
+      if (w0) *o0 = a0;
+      if (w1) *o1 = a1;
+    }
+    cur = nxt;
+    buf ^= 1;
   }
-  if (tx >= cb) return;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int r = ty + 8 * u;
-    if (r >= rb) continue;
-    const long long o = (long long)(r0 + r) * n + c0 + tx;
-    if (i == j) X[o] = acc[u];
-    else B[o] -= acc[u];
-  }
+  cpa_wait<0>();
 }
 
 __global__ void transpose_kernel(const double* in, double* out, int n) {
@@ -229,14 +382,15 @@ __global__ void transpose_kernel(const double* in, double* out, int n) {
   if (x < n && y < n) out[(long long)y * n + x] = t[threadIdx.x][threadIdx.y];
 }
 
-__global__ void symmetrize_kernel(double* A, int n) {
-  long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)n * n) return;
-  int i = (int)(e / n), j = (int)(e % n);
-  if (j >= i) return;
-  double v = 0.5 * (A[(long long)i * n + j] + A[(long long)j * n + i]);
-  A[(long long)i * n + j] = v;
-  A[(long long)j * n + i] = v;
+// out = (in + in^T) / 2
+__global__ void symmetrize_kernel(const double* __restrict__ in, double* __restrict__ out, int n) {
+  __shared__ double t[32][33];
+  int x = blockIdx.y * 32 + threadIdx.x, y = blockIdx.x * 32 + threadIdx.y;
+  if (x < n && y < n) t[threadIdx.y][threadIdx.x] = in[(size_t)y * n + x];
+  __syncthreads();
+  x = blockIdx.x * 32 + threadIdx.x;
+  y = blockIdx.y * 32 + threadIdx.y;
+  if (x < n && y < n) out[(size_t)y * n + x] = 0.5 * (in[(size_t)y * n + x] + t[threadIdx.x][threadIdx.y]);
 }
 
 // ------------------------------------------------------- tridiagonalise ----
@@ -404,13 +558,6 @@ static ofm_status sync_ctx(ofm_ctx* c, const char* what) {
   return OFM_OK;
 }
 
-// X = L^-1 B (n x n) with the multipliers Q of L; B is overwritten.
-static void trsm_lower_left(const double* Q, double* B, double* X, int n, cudaStream_t s) {
-  const int nblk = (n + NB - 1) / NB;
-  for (int j = 0; j < nblk; ++j)
-    trsm_step_kernel<<<dim3(nblk, nblk - j), 256, 0, s>>>(Q, B, X, n, j);
-}
-
 ofm_status ofm_window_factor(ofm_ctx* c) {
   const int n = c->dense_n;
   if (c->fault == OFM_FAULT_NOTPOSDEF) {
@@ -424,25 +571,36 @@ ofm_status ofm_window_factor(ofm_ctx* c) {
   OFM_TRY(ofm_ensure(c, c->w_e, sizeof(double) * n, "window e"));
   OFM_TRY(ofm_ensure(c, c->w_tau, sizeof(double) * n, "window tau"));
   OFM_TRY(ofm_ensure(c, c->w_tmp, sizeof(double) * 2 * n, "window vectors"));
+  const int nblk = (n + NB - 1) / NB, nstr = (n + ST_C - 1) / ST_C;
+  const size_t qbytes = sizeof(double) * (size_t)nblk * NB * NB;
+  OFM_TRY(ofm_ensure(c, c->w_eval, bytes, "window scratch"));
+  OFM_TRY(ofm_ensure(c, c->w_Q, qbytes + 2 * sizeof(int) * nblk, "window multipliers"));
   double* L = (double*)c->w_L.p;
   double* A = (double*)c->w_A.p;
+  double* T = (double*)c->w_eval.p;
+  double* Q = (double*)c->w_Q.p;
+  int* next = (int*)((char*)c->w_Q.p + qbytes);   // item counters, one per launch
   int* flag = (int*)c->flag.p;
   cudaStream_t s = c->stream;
+  OFM_CUDA(c, cudaFuncSetAttribute(factor_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM));
+  OFM_CUDA(c, cudaFuncSetAttribute(reduce_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ST_SMEM));
+  const int sms = 152;
   OFM_CUDA(c, cudaMemcpyAsync(L, c->dense_S.p, bytes, cudaMemcpyDeviceToDevice, s));
+  const dim3 tg((n + 31) / 32, (n + 31) / 32);
+  symmetrize_kernel<<<tg, dim3(32, 32), 0, s>>>((const double*)c->dense_H.p, A, n);
   OFM_CUDA(c, cudaMemsetAsync(flag, 0xff, sizeof(int), s));  // -1: no failure
-  // 1. Cholesky
-  { KTimer kt(c, KC_CHOL, 0, 0.0, (double)n * n * n / 3.0);  // algorithmic n^3/3 flops
-  for (int k0 = 0; k0 < n; k0 += NB) {
-    kt.add(1);
-    const int kb = std::min(NB, n - k0);
-    potrf_diag_kernel<<<1, dim3(32, 32), 0, s>>>(L, n, k0, kb, flag);
-    const int rows = n - k0 - kb;
-    if (rows > 0) {
-      trsm_panel_kernel<<<(rows + 31) / 32, 128, 0, s>>>(L, n, k0, kb);
-      const int tb = (rows + NB - 1) / NB;
-      syrk_update_kernel<<<dim3(tb, tb), dim3(32, 32), 0, s>>>(L, n, k0, kb);
-      kt.add(2);
-    }
+  OFM_CUDA(c, cudaMemsetAsync(next, 0, 2 * sizeof(int) * nblk, s));
+  // 1. S = L L^T, and H -> X = L^-1 H in w_A
+  {
+  KTimer kt(c, KC_CHOL, 2LL * nblk, 0.0, 4.0 / 3.0 * n * n * n);  // n^3/3 of the factor, n^3 of L^-1 H
+  factor_step_kernel<<<1, ST_THREADS, ST_SMEM, s>>>(L, A, Q, n, -1, next, flag);
+  for (int j = 0; j < nblk; ++j) {
+    const int below = std::max(0, n - (j + 1) * NB);
+    panel_kernel<<<(below + 7) / 8 + (n + 7) / 8, 128, 0, s>>>(L, A, Q, n, j);
+    if (below == 0) break;
+    const long long R = nblk - 1 - j, items = R * (R + 1) - 2 + R * nstr;
+    factor_step_kernel<<<(int)std::min<long long>(sms, 1 + items), ST_THREADS, ST_SMEM, s>>>(L, A, Q, n, j, next + j,
+                                                                                          flag);
   }
   }
   OFM_CUDA(c, cudaGetLastError());
@@ -455,24 +613,15 @@ ofm_status ofm_window_factor(ofm_ctx* c) {
     snprintf(buf, sizeof buf, "S is not positive definite: Cholesky pivot %d is not positive", fail);
     return ofm_fail(c, OFM_ERR_NOT_POSDEF, buf);
   }
-  // 2. A = L^-1 H L^-T: multipliers Q of L, X = L^-1 H, then A = L^-1 X^T
-  double* T = (double*)c->dense_H.p;  // kept intact: work on a copy
-  OFM_CUDA(c, cudaMemcpyAsync(A, T, bytes, cudaMemcpyDeviceToDevice, s));
+  // 2. A = L^-1 X^T, from the blocks on and above its diagonal
   {
-  const int nblk = (n + NB - 1) / NB;
-  KTimer kt(c, KC_REDUCE, 5 + 2LL * nblk, 0.0, (double)n * n * n);  // algorithmic (dsygst) n^3 flops
-  OFM_TRY(ofm_ensure(c, c->w_eval, bytes, "window scratch"));
-  OFM_TRY(ofm_ensure(c, c->w_Q, bytes, "window multipliers"));
-  double* X = (double*)c->w_eval.p;
-  double* Q = (double*)c->w_Q.p;
-  inv_diag_kernel<<<nblk, NB, 0, s>>>(L, Q, n);
-  panel_mul_kernel<<<dim3(nblk, nblk), 256, 0, s>>>(L, Q, n);
-  trsm_lower_left(Q, A, X, n, s);          // X = L^-1 H (A is consumed)
-  dim3 tg((n + 31) / 32, (n + 31) / 32);
-  transpose_kernel<<<tg, dim3(32, 32), 0, s>>>(X, A, n);
-  trsm_lower_left(Q, A, X, n, s);          // X = L^-1 (L^-1 H)^T
-  symmetrize_kernel<<<(int)(((long long)n * n + 255) / 256), 256, 0, s>>>(X, n);
-  OFM_CUDA(c, cudaMemcpyAsync(A, X, bytes, cudaMemcpyDeviceToDevice, s));
+  KTimer kt(c, KC_REDUCE, 1 + nblk, 0.0, 1.0 / 3.0 * n * n * n);
+  transpose_kernel<<<tg, dim3(32, 32), 0, s>>>(A, T, n);
+  for (int j = -1; j + 1 < nblk; ++j) {
+    const long long R = j < 0 ? 1 : nblk - 1 - j, S0 = nstr - 2 * (j + 1), items = R * S0 - R * (R - 1);
+    reduce_step_kernel<<<(int)std::min<long long>(sms, items), ST_THREADS, ST_SMEM, s>>>(L, Q, T, A, n, j,
+                                                                                       next + nblk + j + 1);
+  }
   }
   OFM_CUDA(c, cudaGetLastError());
   // 3. tridiagonalise
