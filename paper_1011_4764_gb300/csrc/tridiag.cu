@@ -23,6 +23,7 @@
 #include <cfloat>
 #include <cmath>
 
+#include "fp64_util.h"
 #include "ofm_internal.h"
 
 namespace ofm {
@@ -262,11 +263,11 @@ __device__ __forceinline__ void house_scalars(double x0, double sig, double* hh)
     hh[1] = 0.0;
     hh[2] = 1.0;
   } else {
-    const double nrm = sqrt(fma(x0, x0, sig));
+    const double s2 = fma(x0, x0, sig), nrm = s2 * rsqrt64(s2);
     const double al = (x0 > 0.0) ? -nrm : nrm;
     const double vv = x0 - al;
     hh[0] = al;
-    hh[1] = 2.0 / fma(vv, vv, sig);
+    hh[1] = 2.0 * rcp64(fma(vv, vv, sig));
     hh[2] = vv;
   }
   hh[3] = 0.5 * hh[1];
@@ -474,6 +475,103 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_smem_kernel(double* A, in
     d[n - 1] = fma(-c, v[n - 1], rows[(size_t)((n - 1) / nb) * n + n - 1]);
     e[n - 2] = cl[n - 1];
   }
+}
+
+// The reduction of a small matrix (n <= TS_NMAX) by one CTA of four warps, one
+// per FP64 sub-partition, with A in shared memory.  Per column, warp 0 brings
+// row k+1 up to date and goes on to its norm, alpha and tau while the other
+// warps update their rows and form u = A_k col; then all form p, K and w, each
+// lane its entries.  Bound by the chain of dependent FP64 operations (about 40 of
+// 64 cycles per column), which the exchange between CTAs would lengthen by its
+// two trips through L2: n = 24, 97 us on the CTAs of the whole GPU, 57 here;
+// at n = 96 the rows no longer fit one SM's FP64 rate.
+constexpr int TS_NMAX = 64;
+__global__ void __launch_bounds__(128) tridiag_small_kernel(double* A, int n, double* d, double* e, double* tau) {
+  extern __shared__ double sa[];
+  __shared__ double us[TS_NMAX], rs[TS_NMAX], hs[2][4];   // u, A[i, k+1]; alpha, tau, v0, tau / 2
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ld = n | 1;
+  for (int t = tid; t < n * n; t += 128) sa[(t / n) * ld + t % n] = A[t];
+  __syncthreads();
+  if (warp == 0) named_arrive(1, 128);
+  for (int k = 0; k + 2 < n; ++k) {
+    const double* x = sa + k * ld;   // row k = column k of A_k
+    double* hh = hs[k & 1];
+    double xj[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int j = lane + 32 * q;
+      xj[q] = j > k && j < n ? x[j] : 0.0;
+    }
+    if (warp == 0) {
+      double s = 0.0;
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        if (32 * q + 31 > k + 1 && 32 * q < n) {
+          const double y = lane + 32 * q > k + 1 ? xj[q] : 0.0;
+          s = fma(y, y, s);
+        }
+      s = warp_allsum(s);
+      if (lane == 0) house_scalars(x[k + 1], s, hh);
+    } else {
+      named_sync(1, 128);   // row k and this warp's rows are those of A_k
+      const int sub = lane & 7;
+      for (int i0 = k + 1 + 4 * (warp - 1); i0 < n; i0 += 12) {
+        const int i = i0 + (lane >> 3);
+        const double* row = sa + min(i, n - 1) * ld;
+        double a = 0.0;
+        for (int j = k + 1 + sub; j - sub < n; j += 8)
+          if (j < n) a = fma(row[j], x[j], a);
+        for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (sub == 0 && i < n) {
+          us[i] = a;
+          rs[i] = row[k + 1];
+        }
+      }
+    }
+    __syncthreads();   // u, alpha and tau
+    const double al = hh[0], t = hh[1];
+    double v[2], w[2], s = 0.0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int j = lane + 32 * q;
+      v[q] = w[q] = 0.0;
+      if (32 * q + 31 > k && 32 * q < n) {
+        v[q] = j == k + 1 ? hh[2] : xj[q];
+        if (j > k && j < n) w[q] = t * fma(-al, rs[j], us[j]);
+        s = fma(v[q], w[q], s);
+      }
+    }
+    const double K = hh[3] * warp_allsum(s);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (32 * q + 31 > k && 32 * q < n) w[q] = fma(-K, v[q], w[q]);
+    // rows k+1 (warp 0) and k+2.. (the others): A_ij -= v_i w_j + w_i v_j
+    for (int i = warp == 0 ? k + 1 : k + 1 + warp; i < (warp == 0 ? k + 2 : n); i += 3) {
+      const double vi = __shfl_sync(0xffffffffu, i < 32 ? v[0] : v[1], i & 31);
+      const double wi = __shfl_sync(0xffffffffu, i < 32 ? w[0] : w[1], i & 31);
+      double* row = sa + i * ld;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int j = lane + 32 * q;
+        if (32 * q + 31 > k && 32 * q < n && j > k && j < n) row[j] = fma(-vi, w[q], fma(-wi, v[q], row[j]));
+      }
+    }
+    __syncwarp();
+    if (warp == 0) {
+      if (k + 3 < n) named_arrive(1, 128);   // row k+1 of A_{k+1}
+      for (int q = 0; q < 2; ++q) {
+        const int j = lane + 32 * q;
+        if (j > k && j < n) A[(size_t)k * n + j] = v[q];   // kept for the back-transformation
+      }
+      if (lane == 0) {
+        e[k] = al;
+        tau[k] = t;
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += 128) d[i] = sa[i * ld + i];
+  if (tid == 0) e[n - 2] = sa[(n - 1) * ld + n - 2];
 }
 
 // Number of eigenvalues of the tridiagonal (d, e2 = squared off-diagonals)
@@ -773,6 +871,11 @@ ofm_status ofm_tridiag_persistent(ofm_ctx* c, double* A, int n, double* d, doubl
                                   double* pg) {
   const size_t smem = 2 * (size_t)n * sizeof(double);
   if (n < 3 || smem > 200 * 1024) return OFM_ERR_INVALID;
+  if (n <= TS_NMAX && !c->hold_tri) {   // the held arrival is one of several CTAs
+    tridiag_small_kernel<<<1, 128, (size_t)n * (n | 1) * sizeof(double), c->stream>>>(A, n, d, e, tau);
+    OFM_CUDA(c, cudaGetLastError());
+    return OFM_OK;
+  }
   int dev = 0, coop = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -781,8 +884,10 @@ ofm_status ofm_tridiag_persistent(ofm_ctx* c, double* A, int n, double* d, doubl
   // shared-memory-resident variant when every CTA's rows fit (one CTA per SM)
   {
     // nbs < n: every CTA owns a row below row 0
-    const int nbs = std::min(sms, n - 1);
-    const size_t rmax = (size_t)(n + nbs - 1) / nbs;
+    // the fewest CTAs with as few rows each: more only add readers of every
+    // exchange (n = 315: 1.46 ms on 152 CTAs, 1.38 on 106 with the same three rows)
+    const size_t rmax = (size_t)(n + std::min(sms, n - 1) - 1) / std::min(sms, n - 1);
+    const int nbs = std::min((int)((n + rmax - 1) / rmax), n - 1);
     const size_t smem2 = (rmax * n + 4 * (size_t)n) * sizeof(double);
     const size_t pub_bytes = 4 * (size_t)n * sizeof(Pub);   // p and row k+1, two slots each
     int per_sm2 = 0;
