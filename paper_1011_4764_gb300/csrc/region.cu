@@ -800,13 +800,18 @@ __global__ void __launch_bounds__(RS_THREADS, 1) region_kernel(
 // per item and pass of NP columns it streams the 16-point K chunks of the A
 // pieces (128 stacked state rows) and of the B pieces clipped to the pass
 // into a ring of shared-memory stages with 16-byte asynchronous copies, and
-// each thread accumulates an 8-row x TN-column register tile.  Thread
-// (tr, tc) takes rows 8 (2i + tr/8) + tr%8 and columns 8 (2j + tc/8) + tc%8,
-// so the eight lanes of a quarter warp read one 16-byte unit of A (a
-// broadcast) and eight adjacent units of B (no bank conflict).  Each output
-// is a sum in K order with one FMA per point; the FP32 form stores FP32
-// partial slots (finalized like the tensor-core ones), the FP64 form FP64
-// slots.
+// each thread accumulates a register tile of up to 8 rows x TN columns, columns
+// 8 (2j + tc/8) + tc%8, so that eight lanes read adjacent units of B (no bank
+// conflict) and one of A (a broadcast).  Bound by FP32 / FP64 issue, so what holds
+// no block is left out in steps the registers allow: with more than 96 rows a
+// warp has 16 consecutive ones, one low and one high group to each scheduler, and
+// skips the column quarters where they have no pair (the stacked GEMM needs only
+// fragment pairs a <= b); with fewer the rows are spread over all warps, 2, 4 or 6 to
+// a thread.  27 boxes 31 x 29 x 27, 45 states: FP32 1.66 ms with full 128 x 256
+// tiles, 1.39 now, FP64 38.0 and 29.1; 31 boxes 16 x 32 x 32, 32 states
+// (32 to 96 rows): 0.56 and 0.34, FP64 10.6 and 5.5.  Each output is a sum in K order with
+// one FMA per point; the FP32 form stores FP32 partial slots (finalized like the
+// tensor-core ones), the FP64 form FP64 slots.
 constexpr int SR_THREADS = 256;
 constexpr int SR_NSTAGE = 3;
 
@@ -856,7 +861,7 @@ __global__ void __launch_bounds__(SR_THREADS, 1) region_simt_kernel(
   using V = typename C::V;
   constexpr int G = 512 * C::S;   // bytes of one 8-row group of a chunk
   constexpr int ABYTES = 16 * G, STAGE = ABYTES + (C::NP / 8) * G;
-  constexpr int HT = C::TN / 2;
+  constexpr int QT = C::TN / 4;
   extern __shared__ __align__(16) unsigned char ssm[];
   __shared__ long long s_src[64], s_cb[64];
   __shared__ int s_bytes[64], s_dst[64];
@@ -971,38 +976,67 @@ __global__ void __launch_bounds__(SR_THREADS, 1) region_simt_kernel(
         for (int j = 0; j < C::TN; ++j) acc[i][j] = (T)0;
 #pragma unroll
       for (int ch = 0; ch < SR_NSTAGE - 1; ++ch) issue(ch);
-      for (int ch = 0; ch < nch; ++ch) {
-        issue(ch + SR_NSTAGE - 1);   // into the stage consumed in the previous iteration
-        cpa_wait<SR_NSTAGE - 1>();
-        __syncthreads();
-        const unsigned char* As = ssm + (size_t)(ch % SR_NSTAGE) * STAGE;
-        const unsigned char* Bs = As + ABYTES;
+      // rows of this half; many: 16 consecutive ones per warp, few: spread over the warps
+      const int nrow = s_aend / G * 8;
+      const bool blocks = nrow > 96;
+      const int rb = warp < 4 ? warp : 11 - warp;
+      const int row0 = blocks ? 16 * rb + 8 * (lane >> 4) : tr, rstep = blocks ? 1 : 16;
+      unsigned mask = 0;   // the column quarters in which this warp's rows have a pair
+      if (blocks) {
+        const int rs = s_rrs[128 * hh + 16 * rb + (lane & 15)];
+        if (rs >= 0)
+          for (int q = lane >> 4; q < it.ncs; q += 2) {
+            const RColSeg g = csegs[it.cs0 + q];
+            const int lo = max(g.c0 - c0, 0), hi = min(g.c0 + g.nc - c0, ncp);
+            if (lo < hi && stab[it.st0 + (long long)rs * it.ncf + g.cf] >= 0)
+              for (int jq = lo / (16 * QT); jq <= (hi - 1) / (16 * QT); ++jq) mask |= 1u << jq;
+          }
+        mask = __reduce_or_sync(0xffffffffu, mask);
+      } else {
+        for (int jq = 0; jq < 4; ++jq)
+          if (16 * QT * jq < ncp) mask |= 1u << jq;
+      }
+      auto chunks = [&](auto ri) {
+        constexpr int RI = decltype(ri)::value;   // 8: blocks
+        const int a0 = RI == 8 ? (2 * rb + (lane >> 4)) * G : (tr >> 3) * G + (tr & 7) * 16;
+        constexpr int ASTEP = RI == 8 ? 16 : 2 * G;
+        for (int ch = 0; ch < nch; ++ch) {
+          cpa_wait<SR_NSTAGE - 2>();
+          __syncthreads();             // chunk ch is here; chunk ch - 1 is consumed
+          issue(ch + SR_NSTAGE - 1);   // into the stage of chunk ch - 1
+          const unsigned char* As = ssm + (size_t)(ch % SR_NSTAGE) * STAGE;
+          const unsigned char* Bs = As + ABYTES;
+#pragma unroll 1
+          for (int kc = 0; kc < C::NCORE; ++kc) {
+            V a[RI];
 #pragma unroll
-        for (int kc = 0; kc < C::NCORE; ++kc) {
-          V a[8];
+            for (int i = 0; i < RI; ++i)
+              a[i] = *reinterpret_cast<const V*>(As + a0 + i * ASTEP + kc * 128);
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            a[i] = *reinterpret_cast<const V*>(As + (2 * i + (tr >> 3)) * G + kc * 128 + (tr & 7) * 16);
+            for (int jq = 0; jq < 4; ++jq) {
+              if (!((mask >> jq) & 1u)) continue;   // uniform over the warp
+              V b[QT];
 #pragma unroll
-          for (int jh = 0; jh < 2; ++jh) {
-            V b[HT];
+              for (int j = 0; j < QT; ++j)
+                b[j] = *reinterpret_cast<const V*>(Bs + (2 * (jq * QT + j) + (tc >> 3)) * G + kc * 128 +
+                                                   (tc & 7) * 16);
 #pragma unroll
-            for (int j = 0; j < HT; ++j)
-              b[j] = *reinterpret_cast<const V*>(Bs + (2 * (jh * HT + j) + (tc >> 3)) * G + kc * 128 +
-                                                 (tc & 7) * 16);
+              for (int i = 0; i < RI; ++i)
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-              for (int j = 0; j < HT; ++j) fma_unit(acc[i][jh * HT + j], a[i], b[j]);
+                for (int j = 0; j < QT; ++j) fma_unit(acc[i][jq * QT + j], a[i], b[j]);
+            }
           }
         }
-        __syncthreads();
-      }
+      };
+      if (nrow <= 32) chunks(std::integral_constant<int, 2>());
+      else if (nrow <= 64) chunks(std::integral_constant<int, 4>());
+      else if (nrow <= 96) chunks(std::integral_constant<int, 6>());
+      else chunks(std::integral_constant<int, 8>());
       cpa_wait<0>();
       // epilogue: each valid (row, column) into its pair's slot
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const int row = 128 * hh + 8 * (2 * i + (tr >> 3)) + (tr & 7);
+        const int row = 128 * hh + row0 + i * rstep;
         const int rs = s_rrs[row];
         if (rs < 0) continue;
         const int si = s_ri[row];
