@@ -497,12 +497,15 @@ __global__ void __launch_bounds__(128) tridiag_small_kernel(double* A, int n, do
     const double* x = sa + k * ld;   // row k = column k of A_k
     double* hh = hs[k & 1];
     double xj[2];
+    auto load_row = [&] {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int j = lane + 32 * q;
-      xj[q] = j > k && j < n ? x[j] : 0.0;
-    }
+      for (int q = 0; q < 2; ++q) {
+        const int j = lane + 32 * q;
+        xj[q] = j > k && j < n ? x[j] : 0.0;
+      }
+    };
     if (warp == 0) {
+      load_row();   // this warp wrote row k itself
       double s = 0.0;
 #pragma unroll
       for (int q = 0; q < 2; ++q)
@@ -514,6 +517,7 @@ __global__ void __launch_bounds__(128) tridiag_small_kernel(double* A, int n, do
       if (lane == 0) house_scalars(x[k + 1], s, hh);
     } else {
       named_sync(1, 128);   // row k and this warp's rows are those of A_k
+      load_row();           // not before: warp 0 writes row k after the last CTA barrier
       const int sub = lane & 7;
       for (int i0 = k + 1 + 4 * (warp - 1); i0 < n; i0 += 12) {
         const int i = i0 + (lane >> 3);
