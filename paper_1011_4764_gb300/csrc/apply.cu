@@ -353,7 +353,7 @@ ApplyGrid apply_grid(const std::vector<DevFrag>& fr, bool fp64, int form) {
   if (g.staged) {
     // once per plan (the call is not free: kept out of the launch path)
     const void* k = fp64 ? (const void*)apply_staged_kernel<double> : (const void*)apply_staged_kernel<float>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem) == cudaSuccess)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX) == cudaSuccess)
       return g;
     cudaGetLastError();   // not available: the register form below
     g = ApplyGrid();

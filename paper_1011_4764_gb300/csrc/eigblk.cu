@@ -1129,12 +1129,11 @@ static void gram_plan(const std::vector<EigFrag>& ef, EigGramPlan& g) {
   g.smem = (size_t)std::max<long long>(bytes(g.KP), gmax > 1 ? (long long)GR_THREADS * MI * MI * sizeof(T) : 0);
 }
 
-void eig_gram_plan(const std::vector<EigFrag>& ef, bool fp64, EigGramPlan& g) {
+cudaError_t eig_gram_plan(const std::vector<EigFrag>& ef, bool fp64, EigGramPlan& g) {
   if (fp64) gram_plan<double>(ef, g);
   else gram_plan<float>(ef, g);
   const void* k = fp64 ? (const void*)eig_gram_kernel<double> : (const void*)eig_gram_kernel<float>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) != cudaSuccess)
-    cudaGetLastError();   // the launch reports it
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX);
 }
 
 void launch_eig_gram(const EigGramPlan& g, const EigFrag* d_ef, int nfrag, const int4* d_items,
@@ -1168,12 +1167,11 @@ static void rotate_plan(const std::vector<EigFrag>& ef, int& blocks, size_t& sme
   blocks = std::max(1, std::min(tiles, 4 * 152 / nf));
 }
 
-void eig_rotate_plan(const std::vector<EigFrag>& ef, bool fp64, int& blocks, size_t& smem) {
+cudaError_t eig_rotate_plan(const std::vector<EigFrag>& ef, bool fp64, int& blocks, size_t& smem) {
   if (fp64) rotate_plan<double>(ef, blocks, smem);
   else rotate_plan<float>(ef, blocks, smem);
   const void* k = fp64 ? (const void*)eig_rotate_kernel<double> : (const void*)eig_rotate_kernel<float>;
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    cudaGetLastError();
+  return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX);
 }
 
 void launch_eig_rotate(const EigFrag* d_ef, const DevFrag* d_fr, int nfrag, int blocks, size_t smem,

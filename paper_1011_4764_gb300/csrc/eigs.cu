@@ -827,17 +827,17 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
     w->toff[a] = w->tsum;
     w->tsum += m[a];
   }
-  // the widest block the rotation is built for: its coefficients, a tile of
-  // both blocks and the column sums within an SM's shared memory
-  {
-    const size_t mx = w->mmax, tile = 64;
-    if (256 + (40 + mx * mx + 2 * tile * (mx + 1 + (mx & 1))) * es > 227 * 1024 && (fp64 || mx > 52))
-      return ofm_fail(c, OFM_ERR_INVALID, "block size too large for the rotation kernel");
-  }
+  // the widest block the solver takes: 184 vectors in FP32, 117 in FP64 (at that
+  // width the Gram's stages take 124 KB and the rotation's coefficients and
+  // stages 154 KB)
+  if (w->mmax > (fp64 ? 117 : 184))
+    return ofm_fail(c, OFM_ERR_INVALID, "block size too large for the rotation kernel");
   eig_layout(c->frags, m, w->efr, w->elems, w->vc_elems);
   eig_filter_plan(w->efr, fp64, w->filter);
-  eig_gram_plan(w->efr, fp64, w->gram);
-  eig_rotate_plan(w->efr, fp64, w->rot_blocks, w->rot_smem);
+  OFM_CUDA(c, eig_gram_plan(w->efr, fp64, w->gram));
+  OFM_CUDA(c, eig_rotate_plan(w->efr, fp64, w->rot_blocks, w->rot_smem));
+  if (w->gram.smem > (size_t)SMEM_PLAN_MAX || w->rot_smem > (size_t)SMEM_PLAN_MAX)
+    return ofm_fail(c, OFM_ERR_INVALID, "block size too large for the rotation kernel");
   w->filter_block = w->filter_vc = w->filter_flops = w->gram_bytes = w->gram_flops = w->rot_bytes = w->rot_flops = 0;
   for (int a = 0; a < nf; ++a) {
     const DevFrag& F = c->frags[a];
@@ -882,10 +882,10 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
   w->rr_threads = std::min(fp64 ? rr_max_threads<double>() : rr_max_threads<float>(),
                            std::max(256, 32 * ((w->mmax + 1) / 2)));
   const size_t rr = (3 * (size_t)w->mmax * (w->mmax + 1 + (w->mmax & 1)) + 4 * (size_t)w->mmax) * es;
-  w->rr_smem = rr <= 200 * 1024 ? rr : 0;
+  w->rr_smem = rr <= (size_t)SMEM_PLAN_MAX ? rr : 0;
   if (w->rr_smem) {
-    if (fp64) OFM_CUDA(c, cudaFuncSetAttribute(rayleigh_ritz_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->rr_smem));
-    else OFM_CUDA(c, cudaFuncSetAttribute(rayleigh_ritz_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->rr_smem));
+    if (fp64) OFM_CUDA(c, cudaFuncSetAttribute(rayleigh_ritz_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX));
+    else OFM_CUDA(c, cudaFuncSetAttribute(rayleigh_ritz_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX));
   }
   w->ready = true;
   return OFM_OK;

@@ -143,6 +143,11 @@ void launch_finalize_simt(int prec, const DevFrag* d_fr, const DevPair* d_pairs,
 void launch_scatter_dense(const DevFrag* d_fr, const DevPair* d_pairs, int npairs,
                           const double* blocks, int n, double* Hd, double* Sd, cudaStream_t s);
 
+// Dynamic shared memory a kernel with plan-dependent buffers is allowed.  The
+// limit belongs to the kernel, not to a plan or a context: set to a plan's own
+// size, a smaller plan would take it from the launches of a larger one.
+constexpr int SMEM_PLAN_MAX = 200 * 1024;
+
 // A fragment's block in the eigensolver: state-major vectors of the box's
 // points (eigblk.cu).
 struct EigFrag {
@@ -173,8 +178,8 @@ struct EigGramPlan {
 void eig_layout(const std::vector<DevFrag>& fr, const std::vector<int>& m,
                 std::vector<EigFrag>& out, long long& elems, long long& vc_elems);
 void eig_filter_plan(const std::vector<EigFrag>& ef, bool fp64, EigFilterPlan& plan);
-void eig_gram_plan(const std::vector<EigFrag>& ef, bool fp64, EigGramPlan& plan);
-void eig_rotate_plan(const std::vector<EigFrag>& ef, bool fp64, int& blocks, size_t& smem);
+cudaError_t eig_gram_plan(const std::vector<EigFrag>& ef, bool fp64, EigGramPlan& plan);
+cudaError_t eig_rotate_plan(const std::vector<EigFrag>& ef, bool fp64, int& blocks, size_t& smem);
 void launch_eig_init(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<EigFrag>& ef, void* X,
                      unsigned long long seed, bool fp64, cudaStream_t s);
 void launch_eig_vc(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<EigFrag>& ef, const void* V,

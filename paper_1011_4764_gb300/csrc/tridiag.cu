@@ -907,7 +907,7 @@ static ofm_status arm_hold(ofm_ctx* c) {
 ofm_status ofm_tridiag_persistent(ofm_ctx* c, double* A, int n, double* d, double* e, double* tau,
                                   double* pg) {
   const size_t smem = 2 * (size_t)n * sizeof(double);
-  if (n < 3 || smem > 200 * 1024) return OFM_ERR_INVALID;
+  if (n < 3 || smem > (size_t)SMEM_PLAN_MAX) return OFM_ERR_INVALID;
   if (n <= TS_NMAX && !c->hold_tri) {   // the held arrival is one of several CTAs
     tridiag_small_kernel<<<1, 128, (size_t)n * (n | 1) * sizeof(double), c->stream>>>(A, n, d, e, tau);
     OFM_CUDA(c, cudaGetLastError());
@@ -928,10 +928,10 @@ ofm_status ofm_tridiag_persistent(ofm_ctx* c, double* A, int n, double* d, doubl
     const size_t smem2 = (rmax * n + 4 * (size_t)n) * sizeof(double);
     const size_t pub_bytes = 4 * (size_t)n * sizeof(Pub);   // p and row k+1, two slots each
     int per_sm2 = 0;
-    if (smem2 <= 200 * 1024 && rmax <= (size_t)TRI_RMAX &&
+    if (smem2 <= (size_t)SMEM_PLAN_MAX && rmax <= (size_t)TRI_RMAX &&
         2 * (size_t)n <= (size_t)TRI_PMAX * TRI_THREADS &&
         cudaFuncSetAttribute(tridiag_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem2) == cudaSuccess &&
+                             SMEM_PLAN_MAX) == cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, tridiag_smem_kernel, TRI_THREADS,
                                                       smem2) == cudaSuccess &&
         per_sm2 >= 1 && c->w_eval.cap >= pub_bytes) {
@@ -955,7 +955,7 @@ ofm_status ofm_tridiag_persistent(ofm_ctx* c, double* A, int n, double* d, doubl
     cudaGetLastError();
   }
   OFM_CUDA(c, cudaFuncSetAttribute(tridiag_persistent_kernel,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX));
   int per_sm = 0;
   OFM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_persistent_kernel, 512, smem));
   if (per_sm < 1) return OFM_ERR_INVALID;

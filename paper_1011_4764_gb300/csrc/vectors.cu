@@ -279,7 +279,7 @@ ofm_status ofm_window_vectors(ofm_ctx* c, int m, const double* E, double* C_out)
   const size_t ybytes = sizeof(double) * (size_t)n * m;
   // the factorisations live in shared memory where they fit
   const size_t stmem = (5 * sizeof(double) + 1) * (size_t)n;
-  const bool in_smem = stmem <= 200 * 1024;
+  const bool in_smem = stmem <= (size_t)SMEM_PLAN_MAX;
   const size_t lubytes = in_smem ? 0 : sizeof(double) * 5 * (size_t)n * nc;
   const size_t pivbytes = in_smem ? 0 : ((size_t)n * nc + 15) / 16 * 16;
   const size_t clbytes = sizeof(int) * (size_t)(nc + 1);
@@ -295,15 +295,15 @@ ofm_status ofm_window_vectors(ofm_ctx* c, int m, const double* E, double* C_out)
   {
     KTimer kt(c, KC_VECTORS, 2, 0.0, 4.0 * n * (double)n * m);
     if (in_smem && stmem > 48 * 1024)
-      OFM_CUDA(c, cudaFuncSetAttribute(stein_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stmem));
+      OFM_CUDA(c, cudaFuncSetAttribute(stein_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX));
     stein_kernel<<<nc, 32, in_smem ? stmem : 0, s>>>((const double*)c->w_d.p, (const double*)c->w_e.p, n,
                                                     (const double*)c->w_tmp.p, dcl, tnorm,
                                                     in_smem ? nullptr : lu, piv, Y);
     const size_t row = sizeof(double) * (size_t)n;
-    const bool ring = 6 * row <= 200 * 1024;
+    const bool ring = 6 * row <= (size_t)SMEM_PLAN_MAX;
     const size_t smem = (ring ? 6 : 2) * row;
     const void* bt = ring ? (const void*)backtransform_kernel<4> : (const void*)backtransform_kernel<0>;
-    if (smem > 48 * 1024) OFM_CUDA(c, cudaFuncSetAttribute(bt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) OFM_CUDA(c, cudaFuncSetAttribute(bt, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_PLAN_MAX));
     const double *R = (const double*)c->w_A.p, *tau = (const double*)c->w_tau.p, *L = (const double*)c->w_L.p;
     if (ring) backtransform_kernel<4><<<m, BT_THREADS, smem, s>>>(R, tau, L, n, Y, Cd);
     else backtransform_kernel<0><<<m, BT_THREADS, smem, s>>>(R, tau, L, n, Y, Cd);
