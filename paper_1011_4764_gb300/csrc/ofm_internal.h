@@ -52,11 +52,12 @@ struct Piece {
 };
 
 // Operand planes of one fragment over one box of the grid (a coverage region,
-// or the fragment's own storage box for the pair schedule).
+// or the fragment's own storage box for the pair schedule, whose axis of 8-point
+// units comes first in L, the other two in grid order).
 struct RUnit {
   int frag;
-  int s0[3];          // start (global grid coordinates)
-  int L[3];           // extent
+  int s0[3];          // start (global grid coordinates x, y, z)
+  int L[3];           // extent along the K order's axes, fastest first
   int p8;             // plane stride in K: L[0] * L[1] rounded up to 8
   int ntiles;         // 64-point tiles: (L[2] * p8) / 64 rounded up
   long long tile0;    // first global tile of this unit
@@ -384,7 +385,7 @@ ofm_status ofm_contract_tc(ofm_ctx* c, ofm_precision prec);
 ofm_status ofm_tc_prepare(ofm_ctx* c, ofm_precision prec);   // device tables and buffers
 void ofm_tc_plan_free(struct TcPlan* t);
 ofm_status ofm_pair_planes(ofm_ctx* c, long long bytes, void** arena);
-ofm_status ofm_pair_pack(ofm_ctx* c, int kind, const ofm::RUnit* units, const int4* cta, int ncta,
+ofm_status ofm_pair_pack(ofm_ctx* c, int kind, int axis, const ofm::RUnit* units, const int4* cta, int ncta,
                          void* arena, long long bytes);
 ofm_status ofm_wait_status(ofm_ctx* c);
 // region-stacked contraction (region.cu)

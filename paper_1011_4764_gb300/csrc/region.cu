@@ -61,9 +61,9 @@ namespace {
 // plane, each plane padded to a multiple of 8 points (p8): point (ix, iy, iz)
 // has K index iz * p8 + iy * L[0] + ix, so a 16-byte operand unit (8 BF16 or
 // 4 TF32 points) never straddles two planes.  K is padded to 64-point tiles.
-// The pair schedule packs every fragment's storage box once in the same order,
-// its x range widened to whole 8-point units of the grid (tc.cu): RUnit
-// (ofm_internal.h) describes both.
+// The pair schedule packs every fragment's storage box once in the same way, the
+// axis of its units fastest and widened to whole 8-point units of the grid
+// (tc.cu): RUnit (ofm_internal.h) describes both.
 
 // One contraction work item: up to 256 rows (two 128-row halves sharing the
 // B operand) x an N tile of one region part.
@@ -225,13 +225,15 @@ __device__ __forceinline__ uint32_t rtf32(float x) {
 // CHECK (check mode): every gathered point index is tested against the
 // fragment's dilated box and the states arena, every 16-byte store against
 // the plane arena; a failing access is skipped and *bounds set.
-// PAIR: chunks of one 8-point unit; gxw is the grid's x extent in whole units
-// times 8 (the points past gx do not exist), gx otherwise.
+// PAIR: chunks of one 8-point unit; ua is the axis of the units and guw the
+// grid's extent along it in whole units times 8 (the points past the grid's end
+// do not exist); BF16 hi+lo keeps a unit's two halves together, BF16 uses half
+// of the plan's bytes.
 template <int KIND, bool CHECK = false, bool PAIR = false>
 __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
     const RUnit* __restrict__ units, const int4* __restrict__ cta, const DevFrag* __restrict__ fr,
     const float* __restrict__ V, const float* __restrict__ states, unsigned char* __restrict__ planes,
-    int gx, int gy, int gz, int gxw, double c0d, double c1d, long long n_states, long long n_plane_bytes,
+    int gx, int gy, int gz, int ua, int guw, double c0d, double c1d, long long n_states, long long n_plane_bytes,
     int* bounds) {
   using KT = typename std::conditional<PAIR, PairT<KIND>, KindT<KIND>>::type;
   constexpr int ESZ = KT::esz;
@@ -269,11 +271,14 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
   const int qpp = F.ld / 4;
   const int nq = rows / 4;
   const int npl = U.L[0] * U.L[1];
-  const long long cb = (long long)rows * KT::KC * ESZ;   // bytes of a K chunk
+  constexpr bool UNIT_LO = PAIR && KIND == RK_BF16X3, HALVED = PAIR && KIND == RK_BF16;
+  const long long cb = (long long)rows * KT::KC * ESZ * (UNIT_LO ? 2 : 1);   // bytes of a K chunk
   const long long npl2 = (long long)U.ntiles * 128 * rows;   // one 2-byte plane
-  const long long half = 2 * npl2 * SCL;                     // phi planes -> H phi planes
+  const long long half = (HALVED ? 1 : 2) * npl2 * SCL;      // phi planes -> H phi planes
+  const long long lo = UNIT_LO ? rows * 16 : npl2;           // BF16 hi -> lo
+  const long long base = HALVED ? U.base / 2 : U.base * SCL;
   const int upc = rows * NCORE;                              // units per chunk and plane
-  unsigned char* blk = planes + U.base * SCL;
+  unsigned char* blk = planes + base;
   // phase 1 items (k, q): thread tid starts at item tid and steps by two
   // items of PK_THREADS each (incremental division by nq)
   const int k1s = tid / nq, q1s = tid - k1s * nq;
@@ -296,12 +301,15 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
     bool in = t < job.y + job.z && iz < U.L[2] && r < npl;
     int l[3] = {0, 0, 0}, gi[3] = {0, 0, 0};
     if (in) {
-      const int ii[3] = {r % U.L[0], r / U.L[0], iz};
+      // along the K order's axes (0, 1, 2), (1, 0, 2) or (2, 0, 1) -> x, y, z
+      const int i0 = r % U.L[0], i1 = r / U.L[0];
+      const int ii[3] = {PAIR && ua > 0 ? i1 : i0, !PAIR || ua == 0 ? i1 : ua == 1 ? i0 : iz,
+                         PAIR && ua == 2 ? i0 : iz};
       const int gn[3] = {gx, gy, gz};
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         int g = U.s0[d] + ii[d];
-        const int gw = d == 0 ? gxw : gn[d];
+        const int gw = PAIR && d == ua ? guw : gn[d];
         if (g >= gw) g -= gw;
         if (PAIR && g >= gn[d]) {
           in = false;
@@ -425,8 +433,8 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
       for (int j = 0; j < KPU; ++j) x[j] = src[j * RS];
       const long long off = (long long)(t * KT::CPT + cc) * cb + g * (NCORE * 128) + kc * 128 + r * 16;
       if constexpr (CHECK) {
-        const long long last = U.base * SCL + A * half + off + (KIND == RK_BF16X3 ? npl2 : 0) + 16;
-        if (last > n_plane_bytes || U.base < 0) {
+        const long long last = base + A * half + off + (KIND == RK_BF16X3 ? lo : 0) + 16;
+        if (last > n_plane_bytes || base < 0) {
           atomicExch(bounds, 1);
           continue;
         }
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
         }
         __stcs(reinterpret_cast<uint4*>(blk + A * half + off), make_uint4(hw[0], hw[1], hw[2], hw[3]));
         if constexpr (KIND == RK_BF16X3)
-          __stcs(reinterpret_cast<uint4*>(blk + A * half + npl2 + off), make_uint4(lw[0], lw[1], lw[2], lw[3]));
+          __stcs(reinterpret_cast<uint4*>(blk + A * half + lo + off), make_uint4(lw[0], lw[1], lw[2], lw[3]));
       }
     }
   }   // tiles
@@ -1716,8 +1724,8 @@ ofm_status ofm_region_run(ofm_ctx* c, ofm_precision prec) {
       int* bd = (int*)c->flag.p + OFM_FLAG_BOUNDS;
 #define OFM_PACK(K, CH)                                                                        \
   pack_kernel<K, CH><<<grid, PK_THREADS, sm, c->stream>>>(u, cta, f, V, st, pl, c->grid.n[0],  \
-                                                         c->grid.n[1], c->grid.n[2],         \
-                                                         c->grid.n[0], c0, c1, nst, npb, bd)
+                                                         c->grid.n[1], c->grid.n[2], 0, 0,   \
+                                                         c0, c1, nst, npb, bd)
       const bool ch = c->checks;
       if (kind == RK_TF32) { if (ch) OFM_PACK(RK_TF32, true); else OFM_PACK(RK_TF32, false); }
       else if (kind == RK_BF16) { if (ch) OFM_PACK(RK_BF16, true); else OFM_PACK(RK_BF16, false); }
@@ -1809,7 +1817,7 @@ ofm_status ofm_pair_planes(ofm_ctx* c, long long bytes, void** arena) {
   return OFM_OK;
 }
 
-ofm_status ofm_pair_pack(ofm_ctx* c, int kind, const RUnit* units, const int4* cta, int ncta, void* arena,
+ofm_status ofm_pair_pack(ofm_ctx* c, int kind, int axis, const RUnit* units, const int4* cta, int ncta, void* arena,
                          long long bytes) {
   KTimer t(c, KC_APPLY, 1, c->pack_bytes[kind]);
   const double h = c->grid.h, c0 = 3.0 / (h * h), c1 = 0.5 / (h * h);
@@ -1817,10 +1825,11 @@ ofm_status ofm_pair_pack(ofm_ctx* c, int kind, const RUnit* units, const int4* c
   for (const DevFrag& f : c->frags) maxrows = std::max(maxrows, (f.n + 7) / 8 * 8);
   const int sm = 2 * 64 * ((maxrows + 31) / 32 * 32 + 4) * 4;
   const int* gn = c->grid.n;
+  const int guw = (gn[axis] + 7) / 8 * 8;
 #define OFM_PACKP(K, CH)                                                                              \
   pack_kernel<K, CH, true><<<ncta, PK_THREADS, sm, c->stream>>>(                                      \
       units, cta, (const DevFrag*)c->d_frags.p, (const float*)c->V.p, (const float*)c->states.p,      \
-      (unsigned char*)arena, gn[0], gn[1], gn[2], (gn[0] + 7) / 8 * 8, c0, c1, c->state_elems, bytes, \
+      (unsigned char*)arena, gn[0], gn[1], gn[2], axis, guw, c0, c1, c->state_elems, bytes, \
       (int*)c->flag.p + OFM_FLAG_BOUNDS)
   if (ncta > 0) {
     if (kind == RK_TF32) { if (c->checks) OFM_PACKP(RK_TF32, true); else OFM_PACKP(RK_TF32, false); }

@@ -4,14 +4,15 @@
 // M = n_a (padded to 128), N = 2 n_b (each half padded to 16), K = |R|.
 //
 // Operands.  pack_kernel (region.cu) writes every fragment's states and H phi
-// once per assembly, over its storage box with the x range widened to whole
-// 8-point units of the grid: unit (x/8, y, z) of a fragment is one contiguous
-// block of rows_pad x 8 points in the K-major no-swizzle operand layout (core
-// matrices of 8 states x 16 bytes; TF32 two cores per 8-state group, BF16 one),
-// phi and H phi as separate planes, BF16 hi and lo too.  Both fragments of a
-// pair share the grid's units and are zero outside their own boxes, so the pair
-// sums over the units that both touch, and a run of units along x is one bulk
-// copy per operand: no conversion stands between the copies and the MMAs.  (The
+// once per assembly, over its storage box with one axis widened to whole
+// 8-point units of the grid: a unit (8 points along that axis) of a fragment is
+// one contiguous block of rows_pad x 8 points in the K-major no-swizzle operand
+// layout (core matrices of 8 states x 16 bytes; TF32 two cores per 8-state
+// group, BF16 one; BF16 hi+lo the hi rows, then the lo rows), phi and H phi as
+// separate planes.  Both fragments of a pair share the grid's units and are zero outside their own
+// boxes, so the pair sums over the units that both touch, and a run of units
+// along the axis is one bulk copy per operand: no conversion stands between the
+// copies and the MMAs.  (The
 // form before converted FP32 rows in shared memory, once per pair a fragment is
 // in, through a transposing read: contraction 2.13 ms and H apply 0.12 ms for 56
 // uneven boxes with 826 pairs, TF32; now 0.58 and, with the operands, 0.24 ms.)
@@ -43,10 +44,10 @@ using namespace ofm::ptx;
 namespace {
 
 struct TcFrag {
-  int nux, dext1;     // x units and y extent of the storage box
+  int nux, dext1;     // units along the unit axis, extent along the next axis of the storage box
   int n, rows;        // states, padded to 8
   long long base;     // byte offset in the plane arena
-  long long npl2;     // bytes of one 2-byte plane: hi -> lo, and half of phi -> H phi
+  long long npl2;     // bytes of a plane of 2 bytes per value
 };
 
 struct TcPair {
@@ -57,8 +58,8 @@ struct TcPair {
 
 struct TcItem {
   int pair;
-  int la[3], lb[3];     // start of the piece in both storage boxes (x in units)
-  int m, leny;          // units per row, rows per z plane of the piece
+  int la[3], lb[3];     // start of the piece in both storage boxes, unit axis first (in units)
+  int m, leny;          // units per row, rows per plane of the piece
   int r0, r1;           // rows of the item
   long long part_off;   // FP32 partial tile of n_a x 2 n_b
 };
@@ -66,8 +67,9 @@ struct TcItem {
 enum { TC_TF32 = 0, TC_BF16 = 1, TC_BF16X3 = 2, TC_NKIND = 3 };
 template <int KIND> struct TcKind {
   static constexpr int UB = KIND == TC_TF32 ? 32 : 16;   // bytes of a unit per state
-  static constexpr int NPL = KIND == TC_BF16X3 ? 2 : 1;  // planes per operand
+  static constexpr int NPL = KIND == TC_BF16X3 ? 2 : 1;  // parts of an operand (hi, lo)
   static constexpr int KU = KIND == TC_TF32 ? 1 : 2;     // units per MMA
+  static constexpr int SHARE = KIND == TC_BF16 ? 2 : 1;  // BF16 takes half the plan's bytes
 };
 
 // ----------------------------------------------------------- PTX helpers --
@@ -237,7 +239,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
       const TcItem it = items[ii];
       const TcPair pr = prs[it.pair];
       const TcFrag A = fr[pr.a], B = fr[pr.b];
-      const int ua = A.rows * UB, ub = B.rows * UB;
+      const int ua = A.rows * UB * NPL, ub = B.rows * UB * NPL;   // bytes of a unit
       const int U = tc_units<KIND>(A.rows, B.rows);
       const int nu = (it.r1 - it.r0) * it.m;
       for (int k0 = 0; k0 < nu; k0 += U, ++g) {
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
         }
         const int nk = min(U, nu - k0);
         const uint32_t mb = smem_u32(&full[s]);
-        if (lane == 0) mbar_arrive_expect(mb, (uint32_t)(nk * (ua + 2 * ub) * NPL));
+        if (lane == 0) mbar_arrive_expect(mb, (uint32_t)(nk * (ua + 2 * ub)));
         __syncwarp();
         const int row0 = k0 / it.m, x0 = k0 - row0 * it.m;
         const int nruns = (k0 + nk - 1) / it.m - row0 + 1;   // <= U <= 32
@@ -262,17 +264,14 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
           const int y = r % it.leny, z = r / it.leny;
           const long long qa = ((long long)(it.la[2] + z) * A.dext1 + it.la[1] + y) * A.nux + it.la[0] + x;
           const long long qb = ((long long)(it.lb[2] + z) * B.dext1 + it.lb[1] + y) * B.nux + it.lb[0] + x;
-          const unsigned char* sa = planes + A.base + qa * ua;
-          const unsigned char* sb = planes + B.base + qb * ub;
+          const unsigned char* sa = planes + A.base / KT::SHARE + qa * ua;
+          const unsigned char* sb = planes + B.base / KT::SHARE + qb * ub;
           const uint32_t d = smem_u32(smem + (size_t)s * TS_STAGE);
-          const uint32_t dB = d + (uint32_t)(NPL * U * ua), dH = dB + (uint32_t)(NPL * U * ub);
+          const uint32_t dB = d + (uint32_t)(U * ua), dH = dB + (uint32_t)(U * ub);
           const uint32_t oa = (uint32_t)((ks - k0) * ua), ob = (uint32_t)((ks - k0) * ub);
-#pragma unroll
-          for (int pl = 0; pl < NPL; ++pl) {
-            bulk_g2s(d + (uint32_t)(pl * U * ua) + oa, sa + pl * A.npl2, (uint32_t)(run * ua), mb);
-            bulk_g2s(dB + (uint32_t)(pl * U * ub) + ob, sb + pl * B.npl2, (uint32_t)(run * ub), mb);
-            bulk_g2s(dH + (uint32_t)(pl * U * ub) + ob, sb + (2 + pl) * B.npl2, (uint32_t)(run * ub), mb);
-          }
+          bulk_g2s(d + oa, sa, (uint32_t)(run * ua), mb);
+          bulk_g2s(dB + ob, sb, (uint32_t)(run * ub), mb);
+          bulk_g2s(dH + ob, sb + 2 / KT::SHARE * B.npl2, (uint32_t)(run * ub), mb);
         }
         if (lane == 0) *(volatile int*)&issued_s = g + 1;
       }
@@ -292,7 +291,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
         const TcItem it = items[ii];
         const TcPair pr = prs[it.pair];
         const int ra = fr[pr.a].rows, rb = fr[pr.b].rows;
-        const int ua = ra * UB, ub = rb * UB, U = tc_units<KIND>(ra, rb);
+        const int ua = ra * UB * NPL, ub = rb * UB * NPL, U = tc_units<KIND>(ra, rb);
         const int nu = (it.r1 - it.r0) * it.m;
         const uint32_t N = (uint32_t)((rb + 15) / 16 * 16);
         const uint32_t idesc = instr_desc(FMT, 128, N);
@@ -307,8 +306,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
           const int nk = min(U, nu - k0);
           const uint32_t zero = smem_u32(smem + TS_ZERO);
           uint32_t a = smem_u32(smem + (size_t)s * TS_STAGE);
-          uint32_t p = a + (uint32_t)(NPL * U * ua), h = p + (uint32_t)(NPL * U * ub);
-          const uint32_t la = (uint32_t)(U * ua), lb = (uint32_t)(U * ub);   // hi -> lo
+          uint32_t p = a + (uint32_t)(U * ua), h = p + (uint32_t)(U * ub);
+          const uint32_t la = (uint32_t)(ra * UB), lb = (uint32_t)(rb * UB);   // hi -> lo
           for (int q = 0; q < nk; q += KU) {
             // TF32: both cores of the unit; BF16: this unit's core and the next
             // unit's (zeros after the last)
@@ -461,6 +460,34 @@ void unit_range(int n, int NU, int s, int len, int& us, int& cnt) {
   cnt = std::min(cnt, NU);
 }
 
+// Points (or units) that [oa, oa + ea) and [ob, ob + eb) share on a periodic axis
+// of n.
+long long shared_on_axis(int n, int oa, int ea, int ob, int eb) {
+  const int s = ((ob - oa) % n + n) % n;
+  return std::max(0, std::min(ea, std::min(s + eb, n)) - s) + std::max(0, std::min(ea, s + eb - n));
+}
+
+// Touched units of the boxes along axis d: of the storage box from us (nux of
+// them), of the fragment's own points from us + iu (ic).
+struct UnitAxis {
+  std::vector<int> us, nux, iu, ic;
+  UnitAxis(const std::vector<DevFrag>& fr, int n, int d) {
+    const int NU = (n + 7) / 8;
+    us.resize(fr.size());
+    nux = iu = ic = us;
+    for (size_t f = 0; f < fr.size(); ++f) {
+      const DevFrag& F = fr[f];
+      unit_range(n, NU, F.doff[d], F.dext[d], us[f], nux[f]);
+      iu[f] = 0;
+      ic[f] = NU;
+      if (nux[f] == NU) continue;   // the whole axis: units outside the box hold zeros
+      int s = 0;
+      unit_range(n, NU, (F.doff[d] + F.lo[d]) % n, F.ext[d], s, ic[f]);
+      iu[f] = (s - us[f] + NU) % NU;
+    }
+  }
+};
+
 }  // namespace
 
 struct TcPlan {
@@ -471,6 +498,7 @@ struct TcPlan {
   std::vector<TcItem> items;
   std::vector<int> order;       // items, the largest first
   long long part_elems = 0, plane_bytes = 0;
+  int axis = 0;                 // of the units
   DevBuf d_frags, d_units, d_pcta, d_pairs, d_items, d_order, partials;
   bool ok = false, uploaded = false;
   std::string why;
@@ -513,32 +541,54 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
     t->why = "tensor-core contraction needs FP32 storage";
     return OFM_OK;
   }
-  const int n0 = c->grid.n[0], NU = (n0 + 7) / 8;
-  std::vector<int> us(c->frags.size()), iu(c->frags.size()), ic(c->frags.size());   // storage start; interior units (local)
-  long long tiles = 0;
-  for (size_t f = 0; f < c->frags.size(); ++f) {
-    const DevFrag& F = c->frags[f];
+  for (const DevFrag& F : c->frags)
     if (F.n > 128) {
       t->why = "tensor-core contraction supports at most 128 states per fragment";
       return OFM_OK;
     }
-    TcFrag q;
-    unit_range(n0, NU, F.doff[0], F.dext[0], us[f], q.nux);
-    if (q.nux == NU) {   // the whole axis: units outside the box hold zeros
-      iu[f] = 0;
-      ic[f] = NU;
-    } else {
-      int s = 0;
-      unit_range(n0, NU, (F.doff[0] + F.lo[0]) % n0, F.ext[0], s, ic[f]);
-      iu[f] = (s - us[f] + NU) % NU;
+  // The axis of the units: the one along which the pairs' operand units and the
+  // planes come to the fewest bytes (x among equals).  A box of 18 points at an odd
+  // offset touches four units, 32 points; along an axis that it spans whole, or
+  // shares whole with its neighbours, hardly any point is padding.  Chains along
+  // x in BF16 hi+lo, units always along x and now: 31 boxes of 16 x 32 x 32, 32
+  // states, 308 and 201 us; 64 of 16 x 20 x 32, 16 states, 326 and 216 us; 4 of
+  // 16 x 12 x 12, 6 states, 69 and 55 us (with the unit's hi and lo rows together,
+  // one copy instead of two).
+  const int* gn = c->grid.n;
+  const UnitAxis uax[3] = {UnitAxis(c->frags, gn[0], 0), UnitAxis(c->frags, gn[1], 1), UnitAxis(c->frags, gn[2], 2)};
+  double cost_of[3] = {0, 0, 0};
+  auto rows_of = [&](int f) { return (c->frags[f].n + 7) / 8 * 8; };
+  for (size_t f = 0; f < c->frags.size(); ++f)
+    for (int d = 0; d < 3; ++d)
+      cost_of[d] += 2.0 * rows_of((int)f) * uax[d].nux[f] * c->frags[f].dext[(d + 1) % 3] * c->frags[f].dext[(d + 2) % 3];
+  for (const HostPair& hp : c->pairs) {
+    const DevFrag &A = c->frags[hp.a], &B = c->frags[hp.b];
+    double pts[3], un[3];
+    for (int d = 0; d < 3; ++d) {
+      const UnitAxis& U = uax[d];
+      pts[d] = (double)shared_on_axis(gn[d], A.doff[d] + A.lo[d], A.ext[d], B.doff[d], B.dext[d]);
+      un[d] = (double)shared_on_axis((gn[d] + 7) / 8, U.us[hp.a] + U.iu[hp.a], U.ic[hp.a], U.us[hp.b], U.nux[hp.b]);
     }
-    q.dext1 = F.dext[1];
+    for (int d = 0; d < 3; ++d)
+      cost_of[d] += (rows_of(hp.a) + 2.0 * rows_of(hp.b)) * un[d] * pts[(d + 1) % 3] * pts[(d + 2) % 3];
+  }
+  const int ux = cost_of[1] < cost_of[0] ? (cost_of[2] < cost_of[1] ? 2 : 1) : (cost_of[2] < cost_of[0] ? 2 : 0);
+  const int ax[3] = {ux, ux == 0 ? 1 : 0, ux == 2 ? 1 : 2};   // the K order's axes, fastest first
+  t->axis = ux;
+  const std::vector<int>&us = uax[ux].us, &iu = uax[ux].iu, &ic = uax[ux].ic;
+  const int n0 = gn[ux], NU = (n0 + 7) / 8;
+  long long tiles = 0;
+  for (size_t f = 0; f < c->frags.size(); ++f) {
+    const DevFrag& F = c->frags[f];
+    TcFrag q;
+    q.nux = uax[ux].nux[f];
+    q.dext1 = F.dext[ax[1]];
     q.n = F.n;
-    q.rows = (F.n + 7) / 8 * 8;
+    q.rows = rows_of((int)f);
     RUnit u;
     u.frag = (int)f;
-    u.s0[0] = 8 * us[f]; u.s0[1] = F.doff[1]; u.s0[2] = F.doff[2];
-    u.L[0] = 8 * q.nux; u.L[1] = F.dext[1]; u.L[2] = F.dext[2];
+    for (int d = 0; d < 3; ++d) u.s0[d] = d == ux ? 8 * us[f] : F.doff[d];
+    u.L[0] = 8 * q.nux; u.L[1] = F.dext[ax[1]]; u.L[2] = F.dext[ax[2]];
     u.p8 = u.L[0] * u.L[1];
     u.ntiles = (int)(((long long)u.p8 * u.L[2] + 63) / 64);
     u.tile0 = tiles;
@@ -562,13 +612,16 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
     tq.b = hp.b;
     tq.blk_off = c->simt_pairs[p].blk_off;
     tq.item0 = (int)t->items.size();
-    // x in units, y and z in points
+    // the unit axis in units, the others in points
     std::vector<Run> runs[3];
     runs[0] = dim_runs(NU, (us[hp.a] + iu[hp.a]) % NU, ic[hp.a], us[hp.b], TB.nux);
-    for (int d = 1; d < 3; ++d)
-      runs[d] = dim_runs(c->grid.n[d], (A.doff[d] + A.lo[d]) % c->grid.n[d], A.ext[d], B.doff[d], B.dext[d]);
-    long long xpts = 0, xunits = 0;   // shared points per row, and units they take
-    for (const Run& r : dim_runs(n0, (A.doff[0] + A.lo[0]) % n0, A.ext[0], B.doff[0], B.dext[0])) xpts += r.len;
+    for (int k = 1; k < 3; ++k) {
+      const int d = ax[k];
+      runs[k] = dim_runs(gn[d], (A.doff[d] + A.lo[d]) % gn[d], A.ext[d], B.doff[d], B.dext[d]);
+    }
+    // shared points per row, and units they take
+    const long long xpts = shared_on_axis(n0, A.doff[ux] + A.lo[ux], A.ext[ux], B.doff[ux], B.dext[ux]);
+    long long xunits = 0;
     for (const Run& r : runs[0]) xunits += r.len;
     for (const Run& rz : runs[2])
       for (const Run& ry : runs[1])
@@ -583,7 +636,7 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
           for (int r0 = 0; r0 < rows; r0 += per) {
             TcItem it;
             it.pair = (int)p;
-            it.la[0] = iu[hp.a] + rx.ta; it.la[1] = A.lo[1] + ry.ta; it.la[2] = A.lo[2] + rz.ta;
+            it.la[0] = iu[hp.a] + rx.ta; it.la[1] = A.lo[ax[1]] + ry.ta; it.la[2] = A.lo[ax[2]] + rz.ta;
             it.lb[0] = rx.lb; it.lb[1] = ry.lb; it.lb[2] = rz.lb;
             it.m = rx.len;
             it.leny = ry.len;
@@ -616,13 +669,18 @@ static ofm_status put(ofm_ctx* c, DevBuf& b, const std::vector<T>& v, const char
   return OFM_OK;
 }
 
+// Bytes of the operand planes: 8 per value of the widened boxes (TF32, BF16
+// hi+lo), 4 in BF16.
+static long long arena_bytes(const TcPlan* t, ofm_precision prec) {
+  return std::max<long long>(16, prec == OFM_PREC_BF16 ? t->plane_bytes / 2 : t->plane_bytes);
+}
+
 // Device tables (after a re-plan) and buffers, made before any capture.
 ofm_status ofm_tc_prepare(ofm_ctx* c, ofm_precision prec) {
-  (void)prec;
   TcPlan* t = c->tc;
   if (!t || !t->ok) return ofm_fail(c, OFM_ERR_INVALID, t ? t->why : "no tensor-core plan");
   void* arena = nullptr;
-  OFM_TRY(ofm_pair_planes(c, std::max<long long>(16, t->plane_bytes), &arena));
+  OFM_TRY(ofm_pair_planes(c, arena_bytes(t, prec), &arena));
   OFM_TRY(ofm_ensure_big(c, t->partials, sizeof(float) * (size_t)std::max<long long>(1, t->part_elems), "tc partials"));
   if (t->uploaded) return OFM_OK;
   OFM_TRY(put(c, t->d_frags, t->frags, "tc fragments"));
@@ -651,9 +709,9 @@ ofm_status ofm_contract_tc(ofm_ctx* c, ofm_precision prec) {
   if (!t->uploaded) return ofm_fail(c, OFM_ERR_STATE, "tensor-core plan not prepared");
   const int kind = prec == OFM_PREC_TF32 ? TC_TF32 : prec == OFM_PREC_BF16 ? TC_BF16 : TC_BF16X3;
   void* arena = nullptr;
-  OFM_TRY(ofm_pair_planes(c, std::max<long long>(16, t->plane_bytes), &arena));
-  OFM_TRY(ofm_pair_pack(c, kind, (const RUnit*)t->d_units.p, (const int4*)t->d_pcta.p, (int)t->pack_cta.size(), arena,
-                        t->plane_bytes));
+  OFM_TRY(ofm_pair_planes(c, arena_bytes(t, prec), &arena));
+  OFM_TRY(ofm_pair_pack(c, kind, t->axis, (const RUnit*)t->d_units.p, (const int4*)t->d_pcta.p, (int)t->pack_cta.size(), arena,
+                        arena_bytes(t, prec)));
   int* fl = (int*)c->flag.p + OFM_FLAG_TC;
   int* next = (int*)c->flag.p + OFM_FLAG_QUEUE;
   OFM_CUDA(c, cudaMemsetAsync(next, 0, sizeof(int), c->stream));
