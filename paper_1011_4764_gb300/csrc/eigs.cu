@@ -242,6 +242,18 @@ __device__ __forceinline__ double rsqrt1(double x) {
   const double e = fma(-(x * y), y, 1.0);
   return fma(y * e, fma(e, 0.375, 0.5), y);
 }
+// A pivot's square root and its reciprocal.  In FP32 correctly rounded: a Ritz
+// value of a level tens of Ha deep carries the pivot's relative error (2 u of 88 Ha is
+// 1e-5); in FP64 the fast form.
+__device__ __forceinline__ float pivot_root(float x, float& inv) {
+  const float s = __fsqrt_rn(x);
+  inv = __frcp_rn(s);
+  return s;
+}
+__device__ __forceinline__ double pivot_root(double x, double& inv) {
+  inv = rsqrt1(x);
+  return x * inv;
+}
 __device__ __forceinline__ float madd(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double madd(double a, double b, double c) { return fma(a, b, c); }
 
@@ -394,8 +406,9 @@ __device__ void cta_cholesky(T* M, int m, int ld, T tol, T* rinv, int* ok) {
           T piv = __shfl_sync(0xffffffffu, a[j], j);
           const bool bad = !(piv > tol);
           if (bad) piv = T(1);
-          const T r = rsqrt1(piv);
-          const T x = lane == j ? piv * r : a[j] * r;   // row j of the factor
+          T r;
+          const T d = pivot_root(piv, r);
+          const T x = lane == j ? d : a[j] * r;   // row j of the factor
           if (lane == 0) {
             if (bad) *ok = 0;
             rinv[j0 + j] = r;
@@ -502,6 +515,47 @@ __device__ void rr_row_solves(const T* R, const T* rinv, T* X, int m, int ld) {
   else row_solves<T, 8, BACK>(R, rinv, X, m, ld);   // m <= 256
 }
 
+// val_j = q_j^T B q_j / q_j^T q_j of the rows q_j of Q (m rows of m): a warp takes RB
+// rows at a time, lanes along B's columns.  B need not be symmetric to the last bit.
+template <typename T>
+__device__ void rayleigh_values(const T* B, const T* Q, T* val, int m, int ld) {
+  constexpr int RB = sizeof(T) == 8 ? 2 : 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int r0 = warp * RB; r0 < m; r0 += nw * RB) {
+    const T* q[RB];
+    T s[RB], d[RB];
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+      q[r] = Q + min(r0 + r, m - 1) * ld;
+      s[r] = d[r] = T(0);
+    }
+    for (int k0 = 0; k0 < m; k0 += 32) {
+      const int k = min(k0 + lane, m - 1);
+      T w[RB];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) w[r] = T(0);
+#pragma unroll 4
+      for (int i = 0; i < m; ++i) {
+        const T b = B[i * ld + k];
+#pragma unroll
+        for (int r = 0; r < RB; ++r) w[r] = madd(b, q[r][i], w[r]);
+      }
+      if (k0 + lane < m)
+#pragma unroll
+        for (int r = 0; r < RB; ++r) {
+          s[r] = madd(w[r], q[r][k], s[r]);
+          d[r] = madd(q[r][k], q[r][k], d[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < RB; ++r) {
+      s[r] = warp_sum(s[r]);
+      d[r] = warp_sum(d[r]);
+      if (lane == 0 && r0 + r < m) val[r0 + r] = s[r] / d[r];
+    }
+  }
+}
+
 // At least 256 and at most this many threads (the reduction scratch holds 32
 // warps' partials; the FP64 form needs the registers), one warp per rotation pair of a round where that fits.
 template <typename T>
@@ -521,7 +575,7 @@ __global__ void __launch_bounds__(rr_max_threads<T>()) rayleigh_ritz_kernel(cons
                                                             long long wstride, double* Cm,
                                                             long long cstride, double* theta,
                                                             const long long* toff, double rank_tol,
-                                                            int* rank_out, int use_smem, double v_min) {
+                                                            int* rank_out, int use_smem, double v_min, double tol) {
   extern __shared__ __align__(16) unsigned char rr_raw[];
   __shared__ int perm[520];
   __shared__ T cs[520];
@@ -587,39 +641,66 @@ __global__ void __launch_bounds__(rr_max_threads<T>()) rayleigh_ritz_kernel(cons
       }
       __syncthreads();
       rr_row_solves<T, false>(W, rinv, A, m, ld);
-      // B + sigma I is positive definite: H_f >= min V, with a tenth of B's
-      // largest diagonal entry above it for the rounding of K
+      // sigma: B + sigma I is positive definite.  The larger of two lower bounds
+      // of B's spectrum, Gershgorin's and min V (H_f >= min V), less a tenth of B's
+      // largest diagonal entry for the rounding of K.  The vectors' error is of the
+      // order of u sigma, so sigma follows B, not the potential: with min V alone, a
+      // well anywhere in the grid left its depth times u in every fragment.
+      __syncthreads();
+      for (int i = tid >> 5; i < m; i += nt >> 5) {
+        T s = T(0);
+        for (int j = tid & 31; j < m; j += 32) s += j == i ? T(0) : fabs(A[i * ld + j]);
+        s = warp_sum(s);
+        if ((tid & 31) == 0) sig[i] = A[i * ld + i] - s;
+      }
       __syncthreads();
       if (tid < 32) {
-        T mx = T(0);
-        for (int i = tid; i < m; i += 32) mx = fmax(mx, fabs(A[i * ld + i]));
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        T mx = T(0), low = T(3e38), rad = T(0);
+        for (int i = tid; i < m; i += 32) {
+          const T b = A[i * ld + i];
+          mx = fmax(mx, fabs(b));
+          low = fmin(low, sig[i]);
+          rad = fmax(rad, b - sig[i]);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+          mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+          low = fmin(low, __shfl_xor_sync(0xffffffffu, low, o));
+          rad = fmax(rad, __shfl_xor_sync(0xffffffffu, rad, o));
+        }
         if (tid == 0) {
-          sigma_s = T(0.1) * mx - (T)v_min;
-          chol_ok = 1;
+          sigma_s = T(0.1) * mx - fmax(low, (T)v_min);
+          // The two-sided form instead where sigma is far above B, and on a nearly
+          // diagonal B with a level so deep that the one-sided form's angles, 4 u
+          // each, leave a residual of the order of the tolerance: the two-sided
+          // form's are u |B| over the gap.
+          const bool deep = T(16) * (T)Eps<T>::v * mx > (T)tol && rad <= T(0.05) * mx;
+          chol_ok = sigma_s <= T(4) * mx && !deep;
         }
       }
       __syncthreads();
       const T sigma = sigma_s;
+      const bool shifted = chol_ok != 0;   // uniform
       // U <- the Cholesky factor of B + sigma I (symmetrised), row j = column j
       for (int e = tid; e < m * m; e += nt) {
         const int i = e / m, j = e - (e / m) * m;
         U[i * ld + j] = T(0.5) * (A[i * ld + j] + A[j * ld + i]) + (i == j ? sigma : T(0));
       }
       __syncthreads();
-      cta_cholesky<T>(U, m, ld, T(1e-30), sig, &chol_ok);
+      if (shifted) cta_cholesky<T>(U, m, ld, T(1e-30), sig, &chol_ok);
       bool one = chol_ok != 0;
       if (one) one = jacobi1<T>(U, m, ld, sig, perm);
       if (one) {
-        // lambda_j = |row j|^2 - sigma, Q_j = row j / |row j|
+        // Q_j = row j / |row j|, lambda_j its Rayleigh quotient of B (|row j|^2 - sigma
+        // carries the rounding of every rotation, relative to sigma)
         for (int j = tid >> 5; j < m; j += nt >> 5) {
           T v = T(0);
           for (int i = tid & 31; i < m; i += 32) v = madd(U[j * ld + i], U[j * ld + i], v);
           v = warp_sum(v);
           const T r = rsqrt1(v);
           for (int i = tid & 31; i < m; i += 32) U[j * ld + i] *= r;
-          if ((tid & 31) == 0) sig[j] = v - sigma;
         }
+        __syncthreads();
+        rayleigh_values<T>(A, U, sig, m, ld);
       } else {
         // the two-sided form on B; its vectors, transposed, into U's rows
         for (int e = tid; e < m * m; e += nt) {
@@ -895,7 +976,7 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
 // H X = (H Y) C is formed only for the residual norms, in registers: the
 // next filter starts from X alone and the export reads X, so it is never
 // stored.
-static ofm_status eig_rr(ofm_ctx* c, int y, int hy, int xo, unsigned long long salt) {
+static ofm_status eig_rr(ofm_ctx* c, int y, int hy, int xo, unsigned long long salt, double tol) {
   EigWork* w = c->eig;
   const bool fp64 = c->storage == OFM_STORE_FP64;
   const int nf = c->nfrag;
@@ -913,12 +994,12 @@ static ofm_status eig_rr(ofm_ctx* c, int y, int hy, int xo, unsigned long long s
     rayleigh_ritz_kernel<double><<<nf, w->rr_threads, w->rr_smem, s>>>(
         ef, (const long long*)w->d_gblk.p, (const double*)w->blocks.p,
         (double*)w->work.p, 3 * mm + 4 * w->mmax + 8, (double*)w->Cm.p, mm, (double*)w->theta.p,
-        (const long long*)w->d_toff.p, 1e-13, (int*)w->d_rank.p, w->rr_smem > 0 ? 1 : 0, w->vlim[1]);
+        (const long long*)w->d_toff.p, 1e-13, (int*)w->d_rank.p, w->rr_smem > 0 ? 1 : 0, w->vlim[1], tol);
   else
     rayleigh_ritz_kernel<float><<<nf, w->rr_threads, w->rr_smem, s>>>(
         ef, (const long long*)w->d_gblk.p, (const double*)w->blocks.p,
         (float*)w->work.p, 3 * mm + 4 * w->mmax + 8, (double*)w->Cm.p, mm, (double*)w->theta.p,
-        (const long long*)w->d_toff.p, 1e-5, (int*)w->d_rank.p, w->rr_smem > 0 ? 1 : 0, w->vlim[1]);
+        (const long long*)w->d_toff.p, 1e-5, (int*)w->d_rank.p, w->rr_smem > 0 ? 1 : 0, w->vlim[1], tol);
   }
   KTimer kt(c, KC_ROTATE, 2, w->rot_bytes, w->rot_flops);
   launch_eig_rotate(ef, (const DevFrag*)c->d_frags.p, nf, w->rot_blocks, w->rot_smem, w->buf[y].p, w->buf[hy].p,
@@ -995,7 +1076,7 @@ static ofm_status ofm_fragment_eigs_impl(ofm_ctx* c, const ofm_eig_opts* opts, d
   // initial Rayleigh-Ritz of the random block; xb holds the current block X
   int xb = 0, y = 0, hy = 0;
   OFM_TRY(eig_filter(c, 0, 1, 0, degree, y, hy));
-  OFM_TRY(eig_rr(c, y, hy, 2, 0x1234ULL + o.seed));
+  OFM_TRY(eig_rr(c, y, hy, 2, 0x1234ULL + o.seed, tol));
   xb = 2;
   std::vector<double> th(w->tsum), rs(w->tsum);
   const double bup = 6.0 / (c->grid.h * c->grid.h) + w->vlim[0];
@@ -1088,7 +1169,7 @@ static ofm_status ofm_fragment_eigs_impl(ofm_ctx* c, const ofm_eig_opts* opts, d
     OFM_CUDA(c, cudaMemcpyAsync(w->coef.p, coef.data(), sizeof(double) * 3 * nf * deg, cudaMemcpyHostToDevice, s));
     const int wb = (xb + 1) % 3, xo = (xb + 2) % 3;
     OFM_TRY(eig_filter(c, xb, wb, deg, degree, y, hy));
-    OFM_TRY(eig_rr(c, y, hy, xo, 0x9876ULL * (it + 1) + o.seed));
+    OFM_TRY(eig_rr(c, y, hy, xo, 0x9876ULL * (it + 1) + o.seed, tol));
     xb = xo;
   }
   // export the first n_a Ritz vectors with the sign gauge
