@@ -5,7 +5,7 @@
 // Layout.  A fragment's block is state-major: state j is one contiguous vector
 // of the box's points (EigFrag: the layout's axes are a permutation of the
 // grid's, slowest the longest one the box does not span, its extent along the
-// fastest axis padded to even with zeros).  Each operation then streams whole
+// fastest axis padded to a multiple of four with zeros).  Each operation then streams whole
 // vectors: the filter keeps planes on chip, the Gram and the
 // rotation read and write points with 16-byte accesses and no transposition.
 // The library's states are point-major; init and export convert once per solve.
@@ -409,24 +409,36 @@ __global__ void __launch_bounds__(ft_max(S), 1) eig_filter_kernel(
 }
 
 // One step over HBM, for boxes the kernel above does not take (all three axes
-// spanned, or a large plane): a thread owns one point and eight states; out
-// may be prev (each thread reads its own points of it only).
-template <typename T>
-__global__ void __launch_bounds__(256) eig_step_kernel(const EigFrag* __restrict__ ef, const T* __restrict__ in,
-                                                       const T* prev, T* out,
+// spanned, or a large plane; FP64): a thread owns W consecutive points of the
+// fastest axis and eight states, two at a time; out may be prev (each thread
+// reads its own points of it only).  list: the fragments it is for.  W = 4 in FP32
+// (16-byte accesses: nine per four points and state, one point per thread made
+// that many per point), 1 in FP64, which is bound by the FP64 pipe.
+template <typename T, int W>
+__global__ void __launch_bounds__(256) eig_step_kernel(const EigFrag* __restrict__ ef, const int* __restrict__ list,
+                                                       const T* __restrict__ in, const T* prev, T* out,
                                                        const T* __restrict__ vc,
                                                        const double* __restrict__ coef, T c1) {
-  const EigFrag E = ef[blockIdx.z];
-  const int t = blockIdx.x * 256 + threadIdx.x;
+  struct alignas(W * sizeof(T)) Row {
+    T v[W];
+  };
+  const int f = list[blockIdx.z];
+  const EigFrag E = ef[f];
+  const int t = (blockIdx.x * 256 + threadIdx.x) * W;
   const int j0 = blockIdx.y * 8;
   if (t >= E.Ps || j0 >= E.n) return;
   const int c0 = t % E.e0p, r = t / E.e0p;
   const int c[3] = {c0, r % E.e[1], r / E.e[1]};
-  if (c[0] >= E.e[0] || c[2] >= E.e[2]) return;   // padding stays zero
-  const int st[3] = {1, E.e0p, E.e0p * E.e[1]};
+  const int nv = min(W, E.e[0] - c0);   // valid points; the padding stays zero
+  if (nv <= 0) return;
+  // neighbours: the row before and after along the slower axes, the point before
+  // and after the thread's own along the fastest
   int nb[6];
+  nb[0] = c0 + W < E.e[0] ? t + W : E.full[0] ? t - c0 : -1;
+  nb[1] = c0 > 0 ? t - 1 : E.full[0] ? t + E.e[0] - 1 : -1;
+  const int st[3] = {1, E.e0p, E.e0p * E.e[1]};
 #pragma unroll
-  for (int d = 0; d < 3; ++d)
+  for (int d = 1; d < 3; ++d)
 #pragma unroll
     for (int s = 0; s < 2; ++s) {
       const int q = c[d] + (s ? -1 : 1);
@@ -434,16 +446,54 @@ __global__ void __launch_bounds__(256) eig_step_kernel(const EigFrag* __restrict
                       : E.full[d]          ? t + (s ? (E.e[d] - 1) : (1 - E.e[d])) * st[d]
                                            : -1;
     }
-  const double* cf = coef + 3 * blockIdx.z;
-  const T al = (T)cf[0], be = (T)cf[1], w = al * (vc[E.voff + t] - (T)cf[2]), mc = -al * c1;
-  for (int j = j0; j < min(j0 + 8, E.n); ++j) {
-    const long long b = E.off + (long long)j * E.Ps;
-    T v[6];
+  const double* cf = coef + 3 * f;
+  const T al = (T)cf[0], be = (T)cf[1], mc = -al * c1;
+  T w[W];
+  {
+    const Row v = *reinterpret_cast<const Row*>(vc + E.voff + t);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) v[i] = nb[i] >= 0 ? in[b + nb[i]] : T(0);
-    T o = w * in[b + t];
-    if (prev) o = fma1(be, prev[b + t], o);
-    out[b + t] = fma1(mc, ((v[0] + v[1]) + (v[2] + v[3])) + (v[4] + v[5]), o);
+    for (int i = 0; i < W; ++i) w[i] = al * (v.v[i] - (T)cf[2]);
+  }
+  auto row = [](const T* p, bool ok) {
+    if (ok) return *reinterpret_cast<const Row*>(p);
+    Row z;
+#pragma unroll
+    for (int i = 0; i < W; ++i) z.v[i] = T(0);
+    return z;
+  };
+  constexpr int JB = 2;
+  for (int j = j0; j < min(j0 + 8, E.n); j += JB) {
+    Row x[JB], yp[JB], ym[JB], zp[JB], zm[JB], pv[JB];
+    T xr[JB], xl[JB];
+#pragma unroll
+    for (int u = 0; u < JB; ++u) {
+      const bool on = j + u < E.n;
+      const long long b = E.off + (long long)(on ? j + u : j) * E.Ps;
+      const T* p = in + b;
+      x[u] = row(p + t, true);
+      yp[u] = row(p + nb[2], nb[2] >= 0);
+      ym[u] = row(p + nb[3], nb[3] >= 0);
+      zp[u] = row(p + nb[4], nb[4] >= 0);
+      zm[u] = row(p + nb[5], nb[5] >= 0);
+      xr[u] = nb[0] >= 0 ? p[nb[0]] : T(0);
+      xl[u] = nb[1] >= 0 ? p[nb[1]] : T(0);
+      pv[u] = row(prev + b + t, prev != nullptr);
+    }
+#pragma unroll
+    for (int u = 0; u < JB; ++u) {
+      if (j + u >= E.n) break;
+      Row o;
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const T rt = i + 1 < W && i + 1 < nv ? x[u].v[i + 1 < W ? i + 1 : i] : xr[u];
+        const T lt = i > 0 ? x[u].v[i > 0 ? i - 1 : 0] : xl[u];
+        T v = w[i] * x[u].v[i];
+        if (prev) v = fma1(be, pv[u].v[i], v);
+        v = fma1(mc, ((rt + lt) + (yp[u].v[i] + ym[u].v[i])) + (zp[u].v[i] + zm[u].v[i]), v);
+        o.v[i] = i < nv ? v : T(0);
+      }
+      *reinterpret_cast<Row*>(out + E.off + (long long)(j + u) * E.Ps + t) = o;
+    }
   }
 }
 
@@ -916,7 +966,8 @@ __global__ void __launch_bounds__(256) eig_export_kernel(const EigFrag* ef, cons
 
 // Layout of blocks of m[a] vectors: axes permuted so that the slowest is the
 // longest axis the box does not span (the filter marches along it and its
-// plane is the smallest), the other two in grid order.
+// plane is the smallest), the other two in the order that pads fewer points
+// (a box two points wide is not padded to four), in grid order among equals.
 void eig_layout(const std::vector<DevFrag>& fr, const std::vector<int>& m,
                 std::vector<EigFrag>& out, long long& elems, long long& vc_elems) {
   out.resize(fr.size());
@@ -931,6 +982,8 @@ void eig_layout(const std::vector<DevFrag>& fr, const std::vector<int>& m,
     for (int d = 0; d < 3; ++d)
       if (d != march) E.ax[k++] = d;
     E.ax[2] = march;
+    auto padded = [&](int fast, int next) { return (long long)((F.ext[fast] + 3) / 4 * 4) * F.ext[next]; };
+    if (padded(E.ax[1], E.ax[0]) < padded(E.ax[0], E.ax[1])) std::swap(E.ax[0], E.ax[1]);
     for (int i = 0; i < 3; ++i) {
       E.e[i] = F.ext[E.ax[i]];
       E.full[i] = F.full[E.ax[i]];
@@ -938,7 +991,7 @@ void eig_layout(const std::vector<DevFrag>& fr, const std::vector<int>& m,
     E.e0p = (E.e[0] + 3) / 4 * 4;
     E.Ps = E.e0p * E.e[1] * E.e[2];
     E.n = m[a];
-        E.off = elems;
+    E.off = elems;
     E.voff = vc_elems;
     elems += ((long long)E.Ps * E.n + 63) / 64 * 64;
     vc_elems += ((long long)E.Ps + 63) / 64 * 64;
@@ -963,31 +1016,60 @@ static FilterFn filter_entry(int S, bool even) {
 
 // Work list of the on-chip filter: FP32, boxes that leave an axis to march
 // along and whose plane has at most 448 patches (3584 points); the others go
-// one step per launch (plan.S = 0).  Four levels per launch where two CTAs of
+// one step per launch (plan.steps), beside them, and all of them do where that is
+// faster (filter_prefers_steps).  Four levels per launch where two CTAs of
 // one vector fit an SM (planes of up to about 1400 points), else three, fewer
 // where the shared memory asks for it: per step of 20e6 point-vectors in
 // planes of 32 x 32, S = 4 takes 23 us, S = 3 26 us, S = 2 35 us; of 207e6 in
 // planes of 40 x 40, 275, 250 and 340 us.  Vectors per CTA: the count that keeps
 // the most vectors resident on an SM, the smallest of those (separate CTAs do
 // not wait at each other's barriers).
+//
+// Whether single steps over HBM beat the on-chip filter.  A launch of the latter
+// is a chain of e[2] + S ticks per wave of CTAs, about 0.7 us + 2.3 ns for every
+// thread on the SM each, S steps; a single step is about 6 us and 1.7 us per
+// million point-vectors, 2.7 us past the 8.5 million whose three blocks fit L2.
+// So a few vectors of a long box go by steps: us per step on chip / by steps, 1 box
+// 12 x 12 x 200, 25 vectors 42.6 / 6.3; 100 x 90 x 30, 30 vectors 52 / 20; 8 boxes
+// 24^3, 16 vectors 10.7 / 8.3; but 4 boxes 16 x 12 x 12, 10 vectors 4.5 / 6.3; 8
+// boxes 40^3, 16 vectors 14.6 / 20; 31 boxes 16 x 32 x 32, 40 vectors 25.7 / 55.6.
+static bool filter_prefers_steps(const EigFilterPlan& plan, const std::vector<EigFrag>& ef, long long per_sm) {
+  double total = 0.0;
+  int ticks = 0;
+  for (const int4& j : plan.jobs) {
+    total += 1e-6 * j.z * ef[j.x].Ps;
+    ticks = std::max(ticks, ef[j.x].e[2] + plan.S);
+  }
+  const double ctas = plan.jobs.size() / 152.0, waves = std::max(1.0, ctas / per_sm);
+  const double on_sm = std::max(1.0, std::min(ctas, (double)per_sm));
+  const double chip = waves * ticks / plan.S * (0.7 + 0.0023 * plan.threads * on_sm);
+  return 6.0 + 1.7 * std::min(total, 8.5) + 2.7 * std::max(0.0, total - 8.5) < chip;
+}
+
 void eig_filter_plan(const std::vector<EigFrag>& ef, bool fp64, EigFilterPlan& plan) {
   plan = EigFilterPlan();
-  if (fp64) return;
   const long long cap = 226 * 1024;
   int S = 4;
-  for (const EigFrag& E : ef) {
+  std::vector<char> fits(ef.size(), 0);
+  for (size_t a = 0; a < ef.size(); ++a) {
+    const EigFrag& E = ef[a];
     const long long tp = (long long)(E.e0p / 4) * ((E.e[1] + 1) / 2);
-    if (E.full[2] || tp > ft_max(1)) return;
+    fits[a] = !fp64 && !E.full[2] && tp <= ft_max(1) && filter_smem(E, 1, 1) <= cap;
+    if (!fits[a]) {
+      plan.steps.push_back((int)a);
+      continue;
+    }
     if (2 * ((tp + 31) / 32 * 32) > ft_max(4) || 2 * (filter_smem(E, 1, 4) + 1024) > cap) S = std::min(S, 3);
-    while (S > 0 && filter_smem(E, 1, S) > cap) --S;
+    while (filter_smem(E, 1, S) > cap) --S;
     plan.even = plan.even && E.e[0] % 4 == 0 && E.e[1] % 2 == 0;
   }
-  if (S < 1) return;
+  if (plan.steps.size() == ef.size()) return;
   struct J { int4 j; long long cost; };
   std::vector<J> jobs;
   int threads = 32;
   long long smem = 0;
   for (size_t a = 0; a < ef.size(); ++a) {
+    if (!fits[a]) continue;
     const EigFrag& E = ef[a];
     const int tp = filter_patches(E);
     int np = 1, best = 0;
@@ -1012,12 +1094,28 @@ void eig_filter_plan(const std::vector<EigFrag>& ef, bool fp64, EigFilterPlan& p
   plan.threads = threads;
   plan.smem = (size_t)smem;
   for (const J& j : jobs) plan.jobs.push_back(j.j);
+  const long long per_sm = std::min<long long>(cap / (smem + 1024), ft_max(S) / threads);
+  if (filter_prefers_steps(plan, ef, std::max(1LL, per_sm))) {
+    plan = EigFilterPlan();
+    for (size_t a = 0; a < ef.size(); ++a) plan.steps.push_back((int)a);
+    return;
+  }
   for (int q = 1; q <= S; ++q)
     if (cudaFuncSetAttribute((const void*)filter_entry(q, plan.even), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
       cudaGetLastError();
       plan = EigFilterPlan();
+      for (size_t a = 0; a < ef.size(); ++a) plan.steps.push_back((int)a);
       return;
     }
+}
+
+// Launches of the on-chip filter over L steps.  Every launch, and every single
+// step of the others, swaps the two blocks: where both run, their numbers have
+// the same parity, so that all fragments end in the same block.
+int eig_filter_passes(const EigFilterPlan& plan, int L) {
+  if (plan.S == 0) return 0;
+  const int np = (L + plan.S - 1) / plan.S;
+  return plan.steps.empty() || (np - L) % 2 == 0 ? np : np + 1;   // np + 1 <= L there
 }
 
 static void filter_pass(const EigFilterPlan& plan, const EigFrag* ef, int nfrag, void* A, void* B,
@@ -1029,14 +1127,14 @@ static void filter_pass(const EigFilterPlan& plan, const EigFrag* ef, int nfrag,
 }
 
 int launch_eig_filter(const EigFilterPlan& plan, const EigFrag* d_ef, const std::vector<EigFrag>& ef,
-                      const int4* d_jobs, void* A, void* B, const void* vc, const double* coef, int deg,
-                      int plain_slot, bool fp64, double h, cudaStream_t s, int* launches) {
-  const int nf = (int)ef.size();
-  void *cur = A, *prev = B;   // u_k, u_{k-1}
-  bool hp = false;
-  *launches = 0;
+                      const int4* d_jobs, const int* d_steps, void* A, void* B, const void* vc, const double* coef,
+                      int deg, int plain_slot, bool fp64, double h, cudaStream_t s) {
+  const int nf = (int)ef.size(), L = deg + 1;   // deg steps and H u_deg
+  int swaps = 0;
   if (plan.S > 0) {
-    const int L = deg + 1, np = (L + plan.S - 1) / plan.S;   // deg steps and H u_deg
+    void *cur = A, *prev = B;   // u_k, u_{k-1}
+    bool hp = false;
+    const int np = eig_filter_passes(plan, L);
     for (int i = 0, k = 0; i < np; ++i) {
       const int S = (L - k + (np - i) - 1) / (np - i);
       const bool last = i == np - 1;
@@ -1044,30 +1142,32 @@ int launch_eig_filter(const EigFilterPlan& plan, const EigFrag* d_ef, const std:
       std::swap(cur, prev);   // level S went to prev's block, level S - 1 to cur's
       hp = true;
       k += S;
-      ++*launches;
     }
-  } else {
+    swaps = np;
+  }
+  if (!plan.steps.empty()) {
+    void *cur = A, *prev = B;
     int psmax = 1, rows = 1;
-    for (const EigFrag& E : ef) {
-      psmax = std::max(psmax, E.Ps);
-      rows = std::max(rows, E.n);
+    for (int a : plan.steps) {
+      psmax = std::max(psmax, ef[a].Ps);
+      rows = std::max(rows, ef[a].n);
     }
-    const dim3 g((psmax + 255) / 256, (rows + 7) / 8, nf);
+    const int W = fp64 ? 1 : 4;
+    const dim3 g((psmax / W + 255) / 256, (rows + 7) / 8, (unsigned)plan.steps.size());
     for (int k = 0; k <= deg; ++k) {
       const double* cf = coef + 3 * (size_t)(k == deg ? plain_slot : k) * nf;
-      const bool p = hp && k < deg;
+      const bool p = k > 0 && k < deg;
       if (fp64)
-        eig_step_kernel<double><<<g, 256, 0, s>>>(d_ef, (const double*)cur, p ? (const double*)prev : nullptr,
-                                                  (double*)prev, (const double*)vc, cf, 0.5 / (h * h));
+        eig_step_kernel<double, 1><<<g, 256, 0, s>>>(d_ef, d_steps, (const double*)cur, p ? (const double*)prev : nullptr,
+                                                     (double*)prev, (const double*)vc, cf, 0.5 / (h * h));
       else
-        eig_step_kernel<float><<<g, 256, 0, s>>>(d_ef, (const float*)cur, p ? (const float*)prev : nullptr,
-                                                 (float*)prev, (const float*)vc, cf, (float)(0.5 / (h * h)));
+        eig_step_kernel<float, 4><<<g, 256, 0, s>>>(d_ef, d_steps, (const float*)cur, p ? (const float*)prev : nullptr,
+                                                    (float*)prev, (const float*)vc, cf, (float)(0.5 / (h * h)));
       std::swap(cur, prev);
-      hp = true;
-      ++*launches;
     }
+    swaps = L;
   }
-  return cur == A ? 0 : 1;   // H Y is in A (0) or B (1), Y in the other
+  return swaps & 1;   // H Y is in A (0) or B (1), Y in the other
 }
 
 void launch_eig_init(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<EigFrag>& ef, void* X,

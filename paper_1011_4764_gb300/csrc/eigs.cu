@@ -48,7 +48,7 @@ struct EigWork {
   long long tsum = 0;
   EigFilterPlan filter;
   EigGramPlan gram;
-  DevBuf d_efr, d_jobs, buf[3], vc, coef, theta, res, Cm, work, blocks, partials, d_gitems, d_gpart,
+  DevBuf d_efr, d_jobs, d_steps, buf[3], vc, coef, theta, res, Cm, work, blocks, partials, d_gitems, d_gpart,
       d_gfrag, d_gblk, d_toff, d_rank, d_vmax, rpart, sgn;
   double vlim[2] = {0.0, 0.0};        // max V, min V
   size_t rr_smem = 0, rot_smem = 0;   // dynamic shared memory of the two kernels
@@ -56,9 +56,9 @@ struct EigWork {
   int rot_blocks = 1;
   bool ready = false;
   // algorithmic traffic / work: a launch of the filter that advances S steps
-  // reads one or two blocks and c0 + V and writes two; ten flops per point,
-  // vector and step
-  double filter_block = 0, filter_vc = 0, filter_flops = 0, gram_bytes = 0, gram_flops = 0,
+  // reads one or two blocks and c0 + V and writes two, a single step ([1]) reads
+  // two and writes one; ten flops per point, vector and step
+  double filter_block[2] = {0, 0}, filter_vc[2] = {0, 0}, filter_flops = 0, gram_bytes = 0, gram_flops = 0,
          rot_bytes = 0, rot_flops = 0;
 };
 
@@ -67,6 +67,7 @@ void ofm_eig_guards(const ofm_ctx* c, std::vector<GuardRef>& out) {
   const EigWork* w = c->eig;
   const struct { const DevBuf* b; const char* n; } bufs[] = {
       {&w->d_efr, "eigensolver fragment table"}, {&w->d_jobs, "filter work list"},
+      {&w->d_steps, "filter step list"},
       {&w->buf[0], "eigensolver block 0"}, {&w->buf[1], "eigensolver block 1"},
       {&w->buf[2], "eigensolver block 2"}, {&w->vc, "filter potential"},
       {&w->coef, "filter coefficients"}, {&w->theta, "Ritz values"}, {&w->res, "residuals"},
@@ -82,7 +83,7 @@ void ofm_eig_guards(const ofm_ctx* c, std::vector<GuardRef>& out) {
 void ofm_eig_free(ofm_ctx* c) {
   if (!c->eig) return;
   EigWork* w = c->eig;
-  DevBuf* bufs[] = {&w->d_efr, &w->d_jobs, &w->buf[0], &w->buf[1], &w->buf[2], &w->vc, &w->coef,
+  DevBuf* bufs[] = {&w->d_efr, &w->d_jobs, &w->d_steps, &w->buf[0], &w->buf[1], &w->buf[2], &w->vc, &w->coef,
                     &w->theta, &w->res, &w->Cm, &w->work, &w->blocks, &w->partials, &w->d_gitems,
                     &w->d_gpart, &w->d_gfrag, &w->d_gblk, &w->d_toff, &w->d_rank, &w->d_vmax,
                     &w->rpart, &w->sgn};
@@ -919,12 +920,15 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
   OFM_CUDA(c, eig_rotate_plan(w->efr, fp64, w->rot_blocks, w->rot_smem));
   if (w->gram.smem > (size_t)SMEM_PLAN_MAX || w->rot_smem > (size_t)SMEM_PLAN_MAX)
     return ofm_fail(c, OFM_ERR_INVALID, "block size too large for the rotation kernel");
-  w->filter_block = w->filter_vc = w->filter_flops = w->gram_bytes = w->gram_flops = w->rot_bytes = w->rot_flops = 0;
+  w->filter_block[0] = w->filter_block[1] = w->filter_vc[0] = w->filter_vc[1] = 0;
+  std::vector<char> step(nf, 0);
+  for (int a : w->filter.steps) step[a] = 1;
+  w->filter_flops = w->gram_bytes = w->gram_flops = w->rot_bytes = w->rot_flops = 0;
   for (int a = 0; a < nf; ++a) {
     const DevFrag& F = c->frags[a];
     const double P = (double)F.ext[0] * F.ext[1] * F.ext[2];
-    w->filter_block += P * m[a] * es;
-    w->filter_vc += P * es;
+    w->filter_block[(int)step[a]] += P * m[a] * es;
+    w->filter_vc[(int)step[a]] += P * es;
     w->filter_flops += 10.0 * P * m[a];
     w->gram_bytes += P * 2.0 * m[a] * es;
     w->gram_flops += 2.0 * P * m[a] * 2.0 * m[a];
@@ -951,6 +955,7 @@ static ofm_status eig_setup(ofm_ctx* c, int guard_opt) {
   const struct { DevBuf* b; const void* p; size_t n; const char* what; } tabs[] = {
       {&w->d_efr, w->efr.data(), sizeof(EigFrag) * nf, "eigensolver table"},
       {&w->d_jobs, w->filter.jobs.data(), sizeof(int4) * w->filter.jobs.size(), "filter work list"},
+      {&w->d_steps, w->filter.steps.data(), sizeof(int) * w->filter.steps.size(), "filter step list"},
       {&w->d_gitems, w->gram.items.data(), sizeof(int4) * w->gram.items.size(), "Gram items"},
       {&w->d_gpart, w->gram.part_off.data(), sizeof(long long) * w->gram.part_off.size(), "Gram partial offsets"},
       {&w->d_gfrag, w->gram.fitems.data(), sizeof(int2) * nf, "Gram fragments"},
@@ -1014,15 +1019,18 @@ static ofm_status eig_rr(ofm_ctx* c, int y, int hy, int xo, unsigned long long s
 static ofm_status eig_filter(ofm_ctx* c, int xb, int wb, int deg, int plain_slot, int& y, int& hy) {
   EigWork* w = c->eig;
   const int L = deg + 1;
-  const int passes = w->filter.S > 0 ? (L + w->filter.S - 1) / w->filter.S : L;
+  const int passes = eig_filter_passes(w->filter, L), steps = w->filter.steps.empty() ? 0 : L;
   // the first launch reads one block, the others two; every one writes two
   // (one, when it makes a single step)
   const double blocks = (2.0 * passes - 1.0) + (w->filter.S > 1 ? 2.0 : 1.0) * passes;
-  KTimer kt(c, KC_FILTER, passes, blocks * w->filter_block + passes * w->filter_vc, L * w->filter_flops);
-  int n = 0;
+  KTimer kt(c, KC_FILTER, passes + steps,
+            blocks * w->filter_block[0] + passes * w->filter_vc[0] + (3.0 * L - 1.0) * w->filter_block[1] +
+                L * w->filter_vc[1],
+            L * w->filter_flops);
   const int r = launch_eig_filter(w->filter, (const EigFrag*)w->d_efr.p, w->efr, (const int4*)w->d_jobs.p,
-                                  w->buf[xb].p, w->buf[wb].p, w->vc.p, (const double*)w->coef.p, deg, plain_slot,
-                                  c->storage == OFM_STORE_FP64, c->grid.h, c->stream, &n);
+                                  (const int*)w->d_steps.p, w->buf[xb].p, w->buf[wb].p, w->vc.p,
+                                  (const double*)w->coef.p, deg, plain_slot, c->storage == OFM_STORE_FP64,
+                                  c->grid.h, c->stream);
   hy = r ? wb : xb;
   y = r ? xb : wb;
   OFM_CUDA(c, cudaGetLastError());

@@ -162,11 +162,12 @@ struct EigFrag {
   long long voff;   // first element in the c0 + V arena
 };
 struct EigFilterPlan {
-  int S = 0;              // steps per launch at most; 0: one step per launch over HBM
+  int S = 0;              // steps per launch at most; 0: no fragment takes the on-chip filter
   bool even = true;       // every box splits into whole 4 x 2 patches
   int threads = 0;
   size_t smem = 0;
   std::vector<int4> jobs;
+  std::vector<int> steps; // fragments that go one step per launch over HBM
 };
 struct EigGramPlan {
   std::vector<int4> items;
@@ -188,8 +189,9 @@ void launch_eig_vc(const EigFrag* d_ef, const DevFrag* d_fr, const std::vector<E
 // Filter of degree deg from the block in A (B: workspace, both overwritten),
 // then H Y.  Returns 0 when H Y is in A and Y in B, 1 when the other way round.
 int launch_eig_filter(const EigFilterPlan& plan, const EigFrag* d_ef, const std::vector<EigFrag>& ef,
-                      const int4* d_jobs, void* A, void* B, const void* vc, const double* coef, int deg,
-                      int plain_slot, bool fp64, double h, cudaStream_t s, int* launches);
+                      const int4* d_jobs, const int* d_steps, void* A, void* B, const void* vc, const double* coef,
+                      int deg, int plain_slot, bool fp64, double h, cudaStream_t s);
+int eig_filter_passes(const EigFilterPlan& plan, int L);   // launches of the on-chip filter over L steps
 void launch_eig_gram(const EigGramPlan& g, const EigFrag* d_ef, int nfrag, const int4* d_items,
                      const long long* d_part_off, const int2* d_fitems, const long long* d_blk_off,
                      const void* Y, const void* HY, void* partials, double* blocks, bool fp64, cudaStream_t s);
