@@ -36,6 +36,7 @@
 #include <cstdio>
 #include <vector>
 
+#include "fp64_util.h"
 #include "ofm_internal.h"
 
 using namespace ofm;
@@ -231,18 +232,13 @@ __device__ void cta_jacobi(T* A, T* V, int n, int lda, int* perm, T* cs, double*
   }
 }
 
-// 1 / sqrt(x) to about an ulp for moderate x: the approximate FP32 reciprocal
-// square root and one Newton step, in FP64 one step of the third-order
-// iteration y (1 + e / 2 + 3 e^2 / 8), e = 1 - x y^2 (five FP64 instructions).
+// 1 / sqrt(x) to about an ulp: the approximate FP32 reciprocal square root and one
+// Newton step; rsqrt64 in FP64.
 __device__ __forceinline__ float rsqrt1(float x) {
   const float y = rsqrtf(x);
   return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
-__device__ __forceinline__ double rsqrt1(double x) {
-  const double y = (double)rsqrtf((float)x);
-  const double e = fma(-(x * y), y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
-}
+__device__ __forceinline__ double rsqrt1(double x) { return rsqrt64(x); }
 // A pivot's square root and its reciprocal.  In FP32 correctly rounded: a Ritz
 // value of a level tens of Ha deep carries the pivot's relative error (2 u of 88 Ha is
 // 1e-5); in FP64 the fast form.

@@ -2,9 +2,11 @@
 // warp issues an FP64 instruction every 64 cycles on this part, and the IEEE
 // divide and square root are long sequences of them (1400 cycles together);
 // these start from the FP32 approximation (relative error e of about 1e-7) and
-// make one third-order step, 1 + e + e^2 and 1 + e / 2 + 3 e^2 / 8, whose error
-// is of the order of e^3: within about an ulp.  Arguments whose exponent the FP32
-// range does not hold take the library's divide and square root.
+// make one third-order step of Householder's method, 1 + e + e^2 and
+// 1 + e / 2 + 3 e^2 / 8, whose error is of the order of e^3.  What is left are
+// the roundings of the last operations: at most 0.6 ulp for the reciprocal, 1.1 for
+// the root.  Arguments whose exponent the FP32 range does not hold (zero, infinity
+// and NaN among them) take the library's divide and reciprocal square root.
 #pragma once
 
 #include <cuda_runtime.h>
