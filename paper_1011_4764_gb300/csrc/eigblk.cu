@@ -626,9 +626,14 @@ __global__ void __launch_bounds__(GR_THREADS, sizeof(T) == 4 ? 2 : 3) eig_gram_k
       for (int c = 0; c < MI; ++c) S[(g * MI * MI + r * MI + c) * per + lt] = acc[r][c];
   __syncthreads();
   for (int e = tid; e < MI * MI * per; e += GR_THREADS) {
-    T v = T(0);
-    for (int q = 0; q < G; ++q) v += S[q * MI * MI * per + e];
-    if (e % per < T_) out[e] = v;
+    // four sums side by side: a quarter of the roundings on a large term's sum
+    T v[4] = {T(0), T(0), T(0), T(0)};
+    int q = 0;
+    for (; q + 4 <= G; q += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] += S[(q + u) * MI * MI * per + e];
+    for (; q < G; ++q) v[0] += S[q * MI * MI * per + e];
+    if (e % per < T_) out[e] = (v[0] + v[1]) + (v[2] + v[3]);
   }
 }
 

@@ -239,16 +239,16 @@ __device__ __forceinline__ float rsqrt1(float x) {
   return y * fmaf(-0.5f * x * y, y, 1.5f);
 }
 __device__ __forceinline__ double rsqrt1(double x) { return rsqrt64(x); }
-// A pivot's square root and its reciprocal.  In FP32 correctly rounded: a Ritz
-// value of a level tens of Ha deep carries the pivot's relative error (2 u of 88 Ha is
-// 1e-5); in FP64 the fast form.
+// A pivot's square root and its reciprocal.  In FP32 by correctly rounded
+// operations: Ritz values and vectors of a block with a level tens of Ha deep carry the
+// pivots' relative error (2 u of 88 Ha is 1e-5).
 __device__ __forceinline__ float pivot_root(float x, float& inv) {
   const float s = __fsqrt_rn(x);
   inv = __frcp_rn(s);
   return s;
 }
 __device__ __forceinline__ double pivot_root(double x, double& inv) {
-  inv = rsqrt1(x);
+  inv = rsqrt64(x);
   return x * inv;
 }
 __device__ __forceinline__ float madd(float a, float b, float c) { return fmaf(a, b, c); }
@@ -599,9 +599,13 @@ __global__ void __launch_bounds__(rr_max_threads<T>()) rayleigh_ritz_kernel(cons
     D[i] = g > 0.0 ? (T)(1.0 / sqrt(g)) : T(0);
   }
   __syncthreads();
+  // entry (i, j) of D M D; a diagonal one is rounded once (see pivot_root)
+  auto scaled = [&](double v, int i, int j) {
+    return i == j ? (T)((double)D[i] * D[i] * v) : D[i] * (T)v * D[j];
+  };
   for (int e = tid; e < m * m; e += nt) {
     const int i = e / m, j = e - (e / m) * m;
-    A[i * ld + j] = D[i] * (T)Gb[e] * D[j];
+    A[i * ld + j] = scaled(Gb[e], i, j);
     U[i * ld + j] = (i == j) ? T(1) : T(0);
   }
   __syncthreads();
@@ -626,7 +630,7 @@ __global__ void __launch_bounds__(rr_max_threads<T>()) rayleigh_ritz_kernel(cons
       // solve for; row c of U is then column c of L^-1 (D K D)
       for (int e = tid; e < m * m; e += nt) {
         const int i = e / m, j = e - (e / m) * m;
-        U[i * ld + j] = D[i] * (T)Kb[e] * D[j];
+        U[i * ld + j] = scaled(Kb[e], i, j);
       }
       __syncthreads();
       rr_row_solves<T, false>(W, rinv, U, m, ld);
