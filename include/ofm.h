@@ -189,7 +189,8 @@ ofm_status ofm_assemble_HS(ofm_ctx* ctx, ofm_precision prec, const ofm_assemble_
 /* Result of ofm_autotune_assembly. */
 typedef struct {
   int chunk_points;      /* chosen points per contraction work item (pair schedule) */
-  int stencil_form;      /* chosen form of the H apply: 1 register, 2 staged (shared-memory planes) */
+  int stencil_form;      /* chosen form of the H apply: 1 register, 2 staged (shared-memory planes);
+                            1 for the tensor-core precisions, which run neither */
   double ms;             /* its mean assembly time over the timed runs, milliseconds */
   int n_tried;           /* candidates timed */
   int schedule;          /* chosen schedule: 1 pair, 2 region */
@@ -200,16 +201,18 @@ typedef struct {
 /* Measuring autotuner of the assembly schedule of ofm_assemble_HS (the same
  * computation in every candidate: the schedule moves work between launches
  * and changes the order of the FP32/FP64 partial sums, nothing else).  Each
- * candidate (stencil form 1 or 2) x (points per work item) is planned, run
- * once, then run `reps` times between two CUDA events on the context stream;
- * the fastest becomes the context's schedule, used by later ofm_assemble_HS
+ * candidate (stencil form 1 or 2) x (points per work item) (the latter alone
+ * for the tensor-core precisions) is planned, run once, then run `reps` times
+ * between two CUDA events on the context stream; the fastest becomes the
+ * context's schedule, used by later ofm_assemble_HS
  * calls whose chunk_points is 0, until ofm_build_fragments changes the layout
  * (boxes, state counts, grid or storage).  For the tensor-core precisions
  * the region schedule (ofm_assemble_opts.schedule) is timed too and kept
  * when it is the fastest.  chunks: n_chunks candidate sizes
  * (> 0), or NULL for five: the planner's own size for this precision's
  * contraction times 1/4, 1/2, 1, 2 and 4.  times_ms (host, nullable) gets
- * 2 x n_cand mean times, form-major, -1 where the staged form does not fit.
+ * 2 x n_cand mean times, form-major, -1 where the staged form does not fit
+ * and in its whole row for the tensor-core precisions.
  * out (nullable) gets the choice.  Ends with one assembly of the chosen
  * schedule and synchronises the stream.  Needs states; profiling must be off
  * (OFM_ERR_STATE); reps >= 1 (OFM_ERR_INVALID). */

@@ -867,7 +867,8 @@ extern "C" ofm_status ofm_assemble_HS(ofm_ctx* c, ofm_precision prec, const ofm_
 }
 
 // Measuring autotuner of the assembly schedule: every (stencil form, points
-// per work item) candidate is planned, run once (which captures its graph)
+// per work item) candidate (points per work item alone for the tensor-core
+// precisions) is planned, run once (which captures its graph)
 // and then timed over `reps` runs with CUDA events on the ctx stream; the
 // fastest becomes the ctx's schedule.  The blocks are recomputed with it at
 // the end, so the ctx holds an assembly of the chosen plan.
@@ -913,13 +914,17 @@ extern "C" ofm_status ofm_autotune_assembly(ofm_ctx* c, ofm_precision prec, cons
   const bool tcp = prec >= OFM_PREC_TF32;
   for (int form = 1; form <= 2 && st == OFM_OK; ++form) {
     const ApplyGrid g = apply_grid(c->frags, es == 8, form);
-    const bool fits = form == 1 || g.staged;
+    // the tensor-core precisions run no stencil kernel (the pack forms H phi): one
+    // row of candidates, and the context's stencil stays what it was
+    const bool fits = form == 1 || (g.staged && !tcp);
     for (int i = 0; i < nc && st == OFM_OK; ++i) {
       if (times_ms) times_ms[(form - 1) * nc + i] = -1.0;
       if (!fits) continue;
       drop_graphs(c);
-      c->agrid = g;
-      c->stencil_form = form;
+      if (!tcp) {
+        c->agrid = g;
+        c->stencil_form = form;
+      }
       o.chunk_points = (int)cand[i];
       st = ofm_assemble_HS(c, prec, &o);   // plans, captures and runs once
       if (st != OFM_OK) break;
@@ -978,7 +983,7 @@ extern "C" ofm_status ofm_autotune_assembly(ofm_ctx* c, ofm_precision prec, cons
   // the chosen schedule (the default one after a failure), then one assembly
   // with it
   drop_graphs(c);
-  c->stencil_form = st == OFM_OK ? best_form : 0;
+  if (!tcp) c->stencil_form = st == OFM_OK ? best_form : 0;
   c->tuned_chunk = st == OFM_OK ? best_chunk : 0;
   c->schedule = st == OFM_OK && tcp ? best_sched : 0;
   c->agrid = apply_grid(c->frags, es == 8, c->stencil_form);

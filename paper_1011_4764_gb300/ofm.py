@@ -403,7 +403,9 @@ class Context:
         for the tensor-core precisions, the region schedule, and keeps the
         fastest.  Returns (chunk_points, stencil_form, ms, times) with times a
         (2, n_candidates) array of mean milliseconds (-1: form does not fit);
-        self.tuned holds the schedule chosen and the region time."""
+        self.tuned holds the schedule chosen and the region time.  The
+        tensor-core precisions have no stencil of their own: form 1, and -1 in
+        the second row."""
         cand = None if chunks is None else np.ascontiguousarray(chunks, dtype=np.int32)
         nc = 5 if cand is None else len(cand)
         times = np.full(2 * nc, -1.0)
