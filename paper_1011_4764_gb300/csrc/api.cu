@@ -760,12 +760,12 @@ static ofm_status enqueue_assembly(ofm_ctx* c, ofm_precision prec, int sched) {
     launch_contract_simt(prec, c->storage == OFM_STORE_FP64, (const DevFrag*)c->d_frags.p,
                          (const DevPair*)c->d_pairs.p, (const Piece*)c->d_pieces.p,
                          (const WorkItem*)c->d_items.p, (int)c->simt_items.size(), c->states.p,
-                         c->hphi.p, c->partials.p, c->simt_tile, false, c->stream); }
+                         c->hphi.p, c->partials.p, c->simt_tile, c->stream); }
     OFM_TRY(check_launch(c, "contract (CUDA cores)"));
     { KTimer t(c, KC_FINALIZE, 1, c->finalize_bytes);
     launch_finalize_simt(prec, (const DevFrag*)c->d_frags.p, (const DevPair*)c->d_pairs.p,
                          (int)c->simt_pairs.size(), (const WorkItem*)c->d_items.p, c->partials.p,
-                         c->simt_tile, (double*)c->blocks.p, false, c->stream); }
+                         c->simt_tile, (double*)c->blocks.p, c->stream); }
     OFM_TRY(check_launch(c, "finalize blocks"));
   } else {
     OFM_TRY(ofm_contract_tc(c, prec));

@@ -69,17 +69,13 @@ __device__ __forceinline__ void simt_products(const Tacc* S, int w, int g, int n
 // useful products (tiny chain: 290 us padded, 19 us with these groups).
 // FP64 takes MI = 2 (the finest split, its FMAs hide any shared-memory read),
 // FP32 MI = 4 (2 shared reads per 4 FMAs).
-// upper: for a self pair only the outputs (i, j), i <= j, of both halves are
-// formed (the finalize mirrors them): half the products of a Gram matrix.
 template <typename Tin, typename Tacc, int MI, int NU>
 __global__ void __launch_bounds__(NT) contract_simt_kernel(
     const DevFrag* __restrict__ fr, const DevPair* __restrict__ prs, const Piece* __restrict__ pcs,
     const WorkItem* __restrict__ items, const Tin* __restrict__ states,
-    const Tin* __restrict__ hphi, Tacc* __restrict__ partials, int upper) {
+    const Tin* __restrict__ hphi, Tacc* __restrict__ partials) {
   __shared__ __align__(16) unsigned char stage[STAGE_BYTES];
   __shared__ long long pa_s[KT_MAX], pb_s[KT_MAX];
-  __shared__ unsigned short list[(TILE / MI) * (TILE / MI)];
-  __shared__ int s_T;
 
   const WorkItem it = items[blockIdx.x];
   const DevPair pr = prs[it.pair];
@@ -90,41 +86,15 @@ __global__ void __launch_bounds__(NT) contract_simt_kernel(
   const Tin* Pa = states + A.off;
   const Tin* Pb = states + B.off;
   const Tin* Hb = hphi + B.off;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int lenx = pc.len[0], leny = pc.len[1];
   const int npts = (it.r1 - it.r0) * lenx;
   const int mr = min(TILE, A.n - m0), nc = min(TILE, 2 * B.n - n0);
   const int tm = (mr + MI - 1) / MI, tn = (nc + MI - 1) / MI;
-  const bool half = upper && pr.a == pr.b;
-  if (warp == 0) {
-    // register tiles of the item, row-major; with `half` those that hold an
-    // output on or above the diagonal of either half
-    int cnt = 0;
-    for (int t0 = 0; t0 < tm * tn; t0 += 32) {
-      const int t = t0 + lane;
-      bool need = t < tm * tn;
-      if (need && half) {
-        const int i = m0 + (t / tn) * MI;
-        need = false;
-        for (int q = 0; q < MI; ++q) {
-          const int c = n0 + (t % tn) * MI + q;
-          if (c < 2 * B.n && (c < B.n ? c : c - B.n) >= i) need = true;
-        }
-      }
-      const unsigned b = __ballot_sync(0xffffffffu, need);
-      if (need) list[cnt + __popc(b & ((1u << lane) - 1u))] = (unsigned short)t;
-      cnt += __popc(b);
-    }
-    if (lane == 0) s_T = cnt;
-  }
-  __syncthreads();
-  const int T = s_T;
-  if (T == 0) return;   // a tile below the diagonal: never read (uniform)
+  const int T = tm * tn;   // register tiles of the item, row-major
   const int mrp = tm * MI, ncp = tn * MI, w = mrp + ncp;
   const int ktmax = min(KT_MAX, STAGE_BYTES / (w * (int)sizeof(Tacc)));
-  // at most ktmax groups: a self pair's corner tile can have few register
-  // tiles across wide staged rows
-  const int G = T >= NT ? 1 : min(NT / T, ktmax);
+  const int G = T >= NT ? 1 : min(NT / T, ktmax);   // at most one group per staged point
   const int g = G > 1 ? tid / T : 0;   // >= G: idle in the products
   const int KT = G == 1 ? min(32, ktmax) : G * max(1, min(128, ktmax) / G);
   Tacc* S = reinterpret_cast<Tacc*>(stage);   // [point][A columns, then B columns]
@@ -133,7 +103,7 @@ __global__ void __launch_bounds__(NT) contract_simt_kernel(
 #pragma unroll
   for (int u = 0; u < NU; ++u) {
     const int q = G > 1 ? (u == 0 && g < G ? tid - g * T : T) : tid + u * NT;
-    const int t = q < T ? list[q] : 0;
+    const int t = q < T ? q : 0;
     ra[u] = q < T ? (t / tn) * MI : -1;
     cb[u] = mrp + (t % tn) * MI;
   }
@@ -213,7 +183,7 @@ __global__ void __launch_bounds__(NT) contract_simt_kernel(
   for (int e = tid; e < T * MI * MI; e += NT) {
     Tacc v = Tacc(0);
     for (int q = 0; q < G; ++q) v += S[q * T * MI * MI + e];
-    const int t = list[e % T], ij = e / T;
+    const int t = e % T, ij = e / T;
     out[((t / tn) * MI + ij / MI) * TILE + (t % tn) * MI + ij % MI] = v;
   }
 }
@@ -221,25 +191,24 @@ __global__ void __launch_bounds__(NT) contract_simt_kernel(
 void launch_contract_simt(int prec, bool store_fp64, const DevFrag* d_fr, const DevPair* d_pairs,
                           const Piece* d_pieces, const WorkItem* d_items, int nitems,
                           const void* states, const void* hphi, void* partials, int tile,
-                          bool upper, cudaStream_t s) {
+                          cudaStream_t s) {
   (void)tile;
   if (nitems <= 0) return;
-  const int up = upper ? 1 : 0;
   static_assert(NT * 2 * 2 * sizeof(double) <= STAGE_BYTES && NT * 4 * 4 * sizeof(float) <= STAGE_BYTES,
                 "the groups' sums fit the staging buffer");
   if (prec == OFM_PREC_FP64) {
     if (store_fp64)
       contract_simt_kernel<double, double, 2, 4><<<nitems, NT, 0, s>>>(
           d_fr, d_pairs, d_pieces, d_items, (const double*)states, (const double*)hphi,
-          (double*)partials, up);
+          (double*)partials);
     else
       contract_simt_kernel<float, double, 2, 4><<<nitems, NT, 0, s>>>(
           d_fr, d_pairs, d_pieces, d_items, (const float*)states, (const float*)hphi,
-          (double*)partials, up);
+          (double*)partials);
   } else {
     contract_simt_kernel<float, float, 4, 1><<<nitems, NT, 0, s>>>(
         d_fr, d_pairs, d_pieces, d_items, (const float*)states, (const float*)hphi,
-        (float*)partials, up);
+        (float*)partials);
   }
 }
 
@@ -259,27 +228,21 @@ __device__ __forceinline__ double sum_partials(const DevPair& pr, const WorkItem
 
 // Block layout: H_ab then S_ab, each n_a x n_b row-major; blockIdx.y cuts a
 // pair's outputs (one CTA per pair left the FP64 sums of a few pairs on as
-// many SMs).  upper: a self pair's partials hold only i <= j, mirrored here.
+// many SMs).
 template <typename Tacc>
 __global__ void finalize_simt_kernel(const DevFrag* __restrict__ fr, const DevPair* __restrict__ prs,
                                      const WorkItem* __restrict__ items,
-                                     const Tacc* __restrict__ partials, double* __restrict__ blocks,
-                                     int upper) {
+                                     const Tacc* __restrict__ partials, double* __restrict__ blocks) {
   const DevPair pr = prs[blockIdx.x];
   const int na = fr[pr.a].n, nb = fr[pr.b].n;
   double* Hblk = blocks + pr.blk_off;
   double* Sblk = Hblk + (long long)na * nb;
   const bool diag = (pr.a == pr.b);
   for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < na * nb; e += gridDim.y * blockDim.x) {
-    int i = e / nb, m = e % nb;
-    if (diag && upper && i > m) {
-      const int t = i;
-      i = m;
-      m = t;
-    }
+    const int i = e / nb, m = e % nb;
     double s = sum_partials(pr, items, partials, i, m);
     double h = sum_partials(pr, items, partials, i, nb + m);
-    if (diag && !upper) {
+    if (diag) {
       s = 0.5 * (s + sum_partials(pr, items, partials, m, i));
       h = 0.5 * (h + sum_partials(pr, items, partials, m, nb + i));
     }
@@ -290,17 +253,17 @@ __global__ void finalize_simt_kernel(const DevFrag* __restrict__ fr, const DevPa
 
 void launch_finalize_simt(int prec, const DevFrag* d_fr, const DevPair* d_pairs, int npairs,
                           const WorkItem* d_items, const void* partials, int tile, double* blocks,
-                          bool upper, cudaStream_t s) {
+                          cudaStream_t s) {
   (void)tile;
   if (npairs <= 0) return;
   // about 16 CTAs per SM over all pairs, at most 16 per pair
   const int y = std::min(16, std::max(1, 16 * 152 / npairs));
   if (prec == OFM_PREC_FP64)
     finalize_simt_kernel<double><<<dim3(npairs, y), 256, 0, s>>>(
-        d_fr, d_pairs, d_items, (const double*)partials, blocks, upper ? 1 : 0);
+        d_fr, d_pairs, d_items, (const double*)partials, blocks);
   else
     finalize_simt_kernel<float><<<dim3(npairs, y), 256, 0, s>>>(
-        d_fr, d_pairs, d_items, (const float*)partials, blocks, upper ? 1 : 0);
+        d_fr, d_pairs, d_items, (const float*)partials, blocks);
 }
 
 // Dense basis-ordered matrices from the blocks; the lower block of a pair

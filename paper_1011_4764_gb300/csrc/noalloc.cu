@@ -165,9 +165,9 @@ extern "C" ofm_status ofm_pair_blocks_noalloc(const ofm_grid* grid, const ofm_fr
       (const float*)((intptr_t)hphi_b - (intptr_t)(fr[1].off * (long long)sizeof(float)));
   launch_contract_simt(OFM_PREC_FP32, false, (const DevFrag*)(d + o_fr), (const DevPair*)(d + o_pair),
                        (const Piece*)(d + o_pc), (const WorkItem*)(d + o_it), (int)items.size(),
-                       phi_a, hbase, d + tables, 64, false, s);
+                       phi_a, hbase, d + tables, 64, s);
   launch_finalize_simt(OFM_PREC_FP32, (const DevFrag*)(d + o_fr), (const DevPair*)(d + o_pair), 1,
-                       (const WorkItem*)(d + o_it), d + tables, 64, HS_ab, false, s);
+                       (const WorkItem*)(d + o_it), d + tables, 64, HS_ab, s);
   if (cudaGetLastError() != cudaSuccess) return OFM_ERR_CUDA;
   return OFM_OK;
 }

@@ -137,10 +137,10 @@ void launch_convert_V(const double* src, void* dst, long long n, bool fp64, cuda
 void launch_contract_simt(int prec, bool store_fp64, const DevFrag* d_fr, const DevPair* d_pairs,
                           const Piece* d_pieces, const WorkItem* d_items, int nitems,
                           const void* states, const void* hphi, void* partials, int tile,
-                          bool upper, cudaStream_t s);
+                          cudaStream_t s);
 void launch_finalize_simt(int prec, const DevFrag* d_fr, const DevPair* d_pairs, int npairs,
                           const WorkItem* d_items, const void* partials, int tile,
-                          double* blocks, bool upper, cudaStream_t s);
+                          double* blocks, cudaStream_t s);
 void launch_scatter_dense(const DevFrag* d_fr, const DevPair* d_pairs, int npairs,
                           const double* blocks, int n, double* Hd, double* Sd, cudaStream_t s);
 
