@@ -212,14 +212,38 @@ class ClockSampler:
 
 # ------------------------------------------------------------ oracle legs --
 
-def _sample_pairs(wl, count, seed=0):
-    """A seeded sample of the workload's pairs (self and neighbour pairs)."""
+def _pair_list(grid, frags):
+    """The oracle's pair_list, one vectorised pass per fragment (thousands of
+    boxes in a second)."""
     import numpy as np
-    from paper_1011_4764_gb300 import ofm
-    pairs, cnt, _ = ofm.plan_pairs(wl.grid, wl.frags)
+    from oracle import ofm_oracle as O
+    n = np.array(grid.n)
+    off, ext = np.array([f.off for f in frags]), np.array([f.ext for f in frags])
+    grown = [O.dilated_box(grid, f) for f in frags]
+    goff, gext = np.array([g[0] for g in grown]), np.array([g[1] for g in grown])
+    out = []
+    for a in range(len(frags)):
+        ahead = (goff[a:] - off[a]) % n
+        meet = np.all((ahead < ext[a]) | ((off[a] - goff[a:]) % n < gext[a:]), axis=1)
+        out += [(a, a + int(b)) for b in np.flatnonzero(meet)]
+    return out
+
+
+def _sample_pairs(wl, count, seed=0):
+    """A seeded sample of the workload's pairs (self and neighbour pairs) with the
+    points that their boxes share, the second one grown by a point and not.
+    Of the oracle alone: the reference arm loads nothing of the library."""
+    import numpy as np
+    from oracle import ofm_oracle as O
+    pairs = _pair_list(wl.grid, wl.frags)
     rng = np.random.default_rng(seed)
-    pick = sorted(rng.choice(len(pairs), size=min(count, len(pairs)), replace=False).tolist())
-    return [pairs[i] for i in pick], [tuple(cnt[i]) for i in pick]
+    pick = [pairs[i] for i in sorted(rng.choice(len(pairs), size=min(count, len(pairs)), replace=False).tolist())]
+    cnt = []
+    for a, b in pick:
+        fa, fb = wl.frags[a], wl.frags[b]
+        cnt.append((O.overlap_points(wl.grid, fa.off, fa.ext, fb.off, fb.ext),
+                    O.overlap_points(wl.grid, fa.off, fa.ext, *O.dilated_box(wl.grid, fb)[:2])))
+    return pick, cnt
 
 
 def _oracle_pairs(args):
