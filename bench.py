@@ -719,7 +719,7 @@ def alkane_extra(ofm, stream, dev):
         got = ctx.eigs_by_index(i0, i0 + m)
         d = got - Eo[i0:i0 + m]
         errs[p] = {"max_abs_ha": float(np.max(np.abs(d))), "mean_abs_ha": float(np.mean(np.abs(d))),
-                   "per_eigenvalue_ha": [float(f"{x:.3e}") for x in d]}
+                   "at": _log_levels(f"window errors {p}", d)}
     ctx.close()
     # the all-FP64 path: FP64 states (FP64 eigensolve) and FP64 contraction
     c64 = ofm.Context(stream)
@@ -729,17 +729,27 @@ def alkane_extra(ofm, stream, dev):
     got = c64.eigs_by_index(i0, i0 + m)
     d = got - Eo[i0:i0 + m]
     errs["fp64"] = {"max_abs_ha": float(np.max(np.abs(d))), "mean_abs_ha": float(np.mean(np.abs(d))),
-                    "per_eigenvalue_ha": [float(f"{x:.3e}") for x in d]}
+                    "at": _log_levels("window errors fp64", d)}
     c64.close()
     res["window_error_vs_oracle"] = errs
     return res
 
 
-def _errs(got, ref):
+def _log_levels(what, d):
+    """Every level's error to stderr, a JSON object on its own line (hundreds of
+    them would make the result line too long to read back); returns the index
+    of the largest."""
+    import numpy as np
+    print(json.dumps({"what": what, "per_eigenvalue_ha": [float(f"{x:.3e}") for x in d]}), file=sys.stderr,
+          flush=True)
+    return int(np.argmax(np.abs(d)))
+
+
+def _errs(got, ref, what):
     import numpy as np
     d = got - ref
     return {"max_abs_ha": float(np.max(np.abs(d))), "mean_abs_ha": float(np.mean(np.abs(d))),
-            "per_eigenvalue_ha": [float(f"{x:.3e}") for x in d]}
+            "at": _log_levels(what, d)}
 
 
 def polymer_extra(ofm, stream, dev):
@@ -782,7 +792,8 @@ def polymer_extra(ofm, stream, dev):
         ts.append(e0.elapsed_time(e1))
     res["fp64_full_step_ms"] = min(ts)
     res["window_count"] = int(n)
-    res["window_error_vs_oracle"] = {"fp64": _errs(ctx.eigs_by_index(i0, i0 + m), Eo[i0:i0 + m])}
+    res["window_error_vs_oracle"] = {"fp64": _errs(ctx.eigs_by_index(i0, i0 + m), Eo[i0:i0 + m],
+                                                   "polymer window errors fp64")}
     ctx.close()
     c32 = ofm.Context(stream)
     c32.build_fragments(wl.grid, V_dev, wl.frags, storage="fp32")
@@ -793,7 +804,7 @@ def polymer_extra(ofm, stream, dev):
         try:
             c32.assemble(p)
             res["window_error_vs_oracle"][f"{p}_on_fp32_states"] = _errs(
-                c32.eigs_by_index(i0, i0 + m), Eo[i0:i0 + m])
+                c32.eigs_by_index(i0, i0 + m), Eo[i0:i0 + m], f"polymer window errors {p} on fp32 states")
         except ofm.OFMError as e:
             res["window_error_vs_oracle"][f"{p}_on_fp32_states"] = {"status": str(e)}
     c32.close()
