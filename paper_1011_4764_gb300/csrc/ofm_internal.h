@@ -102,6 +102,7 @@ struct DevBuf {
 // fragments' local coordinates.  Returns (t_start, lb_start, len) triples.
 struct Run { int ta, lb, len; };
 std::vector<Run> dim_runs(int n, int offa, int exta, int offb, int extb);
+long long dim_count(int n, int offa, int exta, int offb, int extb);   // their points
 bool validate_geometry(const ofm_grid& g, const ofm_fragment* f, int nf, std::string& err);
 void make_frag_table(const ofm_grid& g, const ofm_fragment* f, int nf, std::vector<DevFrag>& out,
                      long long& total_elems);

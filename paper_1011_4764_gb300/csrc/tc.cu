@@ -460,13 +460,6 @@ void unit_range(int n, int NU, int s, int len, int& us, int& cnt) {
   cnt = std::min(cnt, NU);
 }
 
-// Points (or units) that [oa, oa + ea) and [ob, ob + eb) share on a periodic axis
-// of n.
-long long shared_on_axis(int n, int oa, int ea, int ob, int eb) {
-  const int s = ((ob - oa) % n + n) % n;
-  return std::max(0, std::min(ea, std::min(s + eb, n)) - s) + std::max(0, std::min(ea, s + eb - n));
-}
-
 // Touched units of the boxes along axis d: of the storage box from us (nux of
 // them), of the fragment's own points from us + iu (ic).
 struct UnitAxis {
@@ -566,8 +559,8 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
     double pts[3], un[3];
     for (int d = 0; d < 3; ++d) {
       const UnitAxis& U = uax[d];
-      pts[d] = (double)shared_on_axis(gn[d], A.doff[d] + A.lo[d], A.ext[d], B.doff[d], B.dext[d]);
-      un[d] = (double)shared_on_axis((gn[d] + 7) / 8, U.us[hp.a] + U.iu[hp.a], U.ic[hp.a], U.us[hp.b], U.nux[hp.b]);
+      pts[d] = (double)dim_count(gn[d], A.doff[d] + A.lo[d], A.ext[d], B.doff[d], B.dext[d]);
+      un[d] = (double)dim_count((gn[d] + 7) / 8, U.us[hp.a] + U.iu[hp.a], U.ic[hp.a], U.us[hp.b], U.nux[hp.b]);
     }
     for (int d = 0; d < 3; ++d)
       cost_of[d] += (rows_of(hp.a) + 2.0 * rows_of(hp.b)) * un[d] * pts[(d + 1) % 3] * pts[(d + 2) % 3];
@@ -620,7 +613,7 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
       runs[k] = dim_runs(gn[d], (A.doff[d] + A.lo[d]) % gn[d], A.ext[d], B.doff[d], B.dext[d]);
     }
     // shared points per row, and units they take
-    const long long xpts = shared_on_axis(n0, A.doff[ux] + A.lo[ux], A.ext[ux], B.doff[ux], B.dext[ux]);
+    const long long xpts = dim_count(n0, A.doff[ux] + A.lo[ux], A.ext[ux], B.doff[ux], B.dext[ux]);
     long long xunits = 0;
     for (const Run& r : runs[0]) xunits += r.len;
     for (const Run& rz : runs[2])
