@@ -99,8 +99,12 @@ typedef struct {
                             schedule (the one ofm_autotune_assembly chose), else, and for
                             FP32 / FP64, "region" where its plan applies and its MMA
                             work, padding included, stays within 4x the algorithmic
-                            flops, else "pair"; 1 "pair": H phi in the states' layout,
-                            then one GEMM per pair (M = n_a padded to 128); 2 "region":
+                            flops, else "pair"; 1 "pair": one GEMM per pair (M = n_a
+                            padded to 128 on the tensor cores, whose operands, states and
+                            H phi, are packed once per fragment; FP32 and FP64 form H phi
+                            in the states' layout and multiply the valid outputs only,
+                            which is the faster of their two schedules: ask for it where
+                            their time matters); 2 "region":
                             the grid is cut into coverage regions (products of the
                             segments between dilated-box boundaries) and every region's
                             fragments are stacked into one GEMM (M = sum of their
