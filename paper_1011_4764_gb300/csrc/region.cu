@@ -227,8 +227,8 @@ __device__ __forceinline__ uint32_t rtf32(float x) {
 // the plane arena; a failing access is skipped and *bounds set.
 // PAIR: chunks of one 8-point unit; ua is the axis of the units and guw the
 // grid's extent along it in whole units times 8 (the points past the grid's end
-// do not exist); BF16 hi+lo keeps a unit's two halves together, BF16 uses half
-// of the plan's bytes.
+// do not exist); a unit keeps its parts together, BF16 uses half of the plan's
+// bytes.
 template <int KIND, bool CHECK = false, bool PAIR = false>
 __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
     const RUnit* __restrict__ units, const int4* __restrict__ cta, const DevFrag* __restrict__ fr,
@@ -271,12 +271,12 @@ __global__ void __launch_bounds__(PK_THREADS, 3) pack_kernel(
   const int qpp = F.ld / 4;
   const int nq = rows / 4;
   const int npl = U.L[0] * U.L[1];
-  constexpr bool UNIT_LO = PAIR && KIND == RK_BF16X3, HALVED = PAIR && KIND == RK_BF16;
-  const long long cb = (long long)rows * KT::KC * ESZ * (UNIT_LO ? 2 : 1);   // bytes of a K chunk
+  constexpr int PARTS = !PAIR ? 1 : KIND == RK_BF16X3 ? 4 : 2;   // of a chunk: phi, H phi (hi), then lo
+  const long long cb = (long long)rows * KT::KC * ESZ * PARTS;   // bytes of a K chunk
   const long long npl2 = (long long)U.ntiles * 128 * rows;   // one 2-byte plane
-  const long long half = (HALVED ? 1 : 2) * npl2 * SCL;      // phi planes -> H phi planes
-  const long long lo = UNIT_LO ? rows * 16 : npl2;           // BF16 hi -> lo
-  const long long base = HALVED ? U.base / 2 : U.base * SCL;
+  const long long half = PAIR ? cb / PARTS : 2 * npl2 * SCL; // phi -> H phi
+  const long long lo = PAIR ? 2 * half : npl2;               // BF16 hi -> lo
+  const long long base = PAIR && KIND == RK_BF16 ? U.base / 2 : U.base * SCL;
   const int upc = rows * NCORE;                              // units per chunk and plane
   unsigned char* blk = planes + base;
   // phase 1 items (k, q): thread tid starts at item tid and steps by two

@@ -1,21 +1,24 @@
 // Pair-block contraction on the 5th-generation tensor cores (tcgen05), the
 // "pair" schedule:
 //     [S_ab | H_ab] = Phi_a[R]^T [Phi_b[R] | HPhi_b[R]]   (Sec. II),
-// M = n_a (padded to 128), N = 2 n_b (each half padded to 16), K = |R|.
+// M = n_a (padded to 128), N = 2 n_b (each half padded to 8), K = |R|.
 //
 // Operands.  pack_kernel (region.cu) writes every fragment's states and H phi
 // once per assembly, over its storage box with one axis widened to whole
 // 8-point units of the grid: a unit (8 points along that axis) of a fragment is
 // one contiguous block of rows_pad x 8 points in the K-major no-swizzle operand
 // layout (core matrices of 8 states x 16 bytes; TF32 two cores per 8-state
-// group, BF16 one; BF16 hi+lo the hi rows, then the lo rows), phi and H phi as
-// separate planes.  Both fragments of a pair share the grid's units and are zero outside their own
-// boxes, so the pair sums over the units that both touch, and a run of units
-// along the axis is one bulk copy per operand: no conversion stands between the
-// copies and the MMAs.  (The
-// form before converted FP32 rows in shared memory, once per pair a fragment is
-// in, through a transposing read: contraction 2.13 ms and H apply 0.12 ms for 56
-// uneven boxes with 826 pairs, TF32; now 0.58 and, with the operands, 0.24 ms.)
+// group, BF16 one), the rows of phi and of H phi one after the other (BF16 hi+lo:
+// both hi, then both lo): one operand of 2 rows_pad MMA columns, since an MMA of 128
+// rows takes the same 33 ns for any number of them.  Both fragments of a pair share
+// the grid's units and are zero outside their own boxes, so the pair sums over the
+// units that both touch, and a run of units along the axis is one bulk copy: no
+// conversion stands between the copies and the MMAs.  Of a only phi is wanted: its
+// units come whole, H phi too (one copy a run, some 40 ns each, instead of one or two
+// a unit), where they are small; a pair of a fragment with itself takes a's rows
+// from b's copy.  56 uneven boxes with 826 pairs: contraction 2.13 ms in TF32 and 1.69
+// in BF16 hi+lo with a conversion of FP32 rows in shared memory for every pair, 0.58
+// and 0.74 ms with phi and H phi as separate planes and MMAs, 0.53 and 0.56 ms now.
 //
 // A persistent CTA per SM takes items (pair, rows of units of a piece) from a
 // global counter, the largest first, through a warp-specialised pipeline: a
@@ -23,8 +26,8 @@
 // thread issues the MMAs into two alternating TMEM accumulators (a K step is one
 // unit in TF32, two in BF16; hi*hi + hi*lo + lo*hi for the split), four warps
 // drain an accumulator into the item's FP32 partial tile.  Operand rows past a
-// fragment's own (M to 128, N to 16) are whatever follows in shared memory:
-// they reach only accumulator rows and columns that nobody reads.  A finalize
+// fragment's own (M to 128) are whatever follows in shared memory: they reach
+// only accumulator rows that nobody reads.  A finalize
 // kernel sums the partials of each pair in a fixed order.  Every wait is
 // bounded: on timeout the CTA sets an error flag, drains its copies and MMAs,
 // frees its tensor memory and returns.
@@ -47,7 +50,6 @@ struct TcFrag {
   int nux, dext1;     // units along the unit axis, extent along the next axis of the storage box
   int n, rows;        // states, padded to 8
   long long base;     // byte offset in the plane arena
-  long long npl2;     // bytes of a plane of 2 bytes per value
 };
 
 struct TcPair {
@@ -143,19 +145,35 @@ constexpr int TS_STAGE = 48 * 1024;
 constexpr int TS_UMAX = 32;           // units of a stage at most (one run per lane)
 constexpr int TS_NQ = 4;              // work-item ring between the roles
 constexpr int TS_ACC_COLS = 256;      // TMEM columns of one accumulator; two of them
-// stages, then room for the operand rows read past the last one, then 2 KB of
-// zeros (the second half of a BF16 K step whose item ends with a single unit)
-constexpr int TS_SLACK = 8 * 1024, TS_ZERO = TS_NSTAGE * TS_STAGE + TS_SLACK, TS_SMEM = TS_ZERO + 2048;
+// stages, then room for the operand rows read past the last one, then 4 KB of
+// zeros: the second half of a BF16 K step whose item ends with a single unit, 16
+// bytes for each of up to 256 rows
+constexpr int TS_NZERO = 256 * 16;
+constexpr int TS_SLACK = 8 * 1024, TS_ZERO = TS_NSTAGE * TS_STAGE + TS_SLACK, TS_SMEM = TS_ZERO + TS_NZERO;
 
 // Units per stage of a pair: a stage holds the units of both operands' planes;
 // even, so that only an item's last stage can end with half a BF16 K step.
 constexpr int TS_MINUNITS = 256;       // units an item may take whatever part of them is padding
-template <int KIND>
-__host__ __device__ constexpr int tc_units(int ra, int rb) {
-  const int u = TS_STAGE / ((ra + 2 * rb) * TcKind<KIND>::UB * TcKind<KIND>::NPL);
-  return u > TS_UMAX ? TS_UMAX : u / 2 * 2;
-}
-static_assert(tc_units<TC_TF32>(128, 128) >= 2 && tc_units<TC_BF16X3>(128, 128) >= 2, "two units fit a stage");
+
+// A pair's units in shared memory: bytes of a unit of b (phi, H phi), of a (the
+// same, phi alone, or none of its own) and a's lo rows after its hi rows.  a comes
+// whole where a stage still holds four units of both (BF16 hi+lo: 8 boxes 40^3, 96
+// states, 612 us whole, 687 by parts; 27 boxes 24^3, 128 states, two units a stage,
+// 926 and 836).
+template <int KIND> struct TcShape {
+  int pa, wa, wb, sa, lo_a, units;
+  bool self, whole;
+  __host__ __device__ constexpr TcShape(int ra, int rb, bool same)
+      : pa(ra * TcKind<KIND>::UB), wa(2 * TcKind<KIND>::NPL * pa), wb(2 * TcKind<KIND>::NPL * rb * TcKind<KIND>::UB),
+        sa(0), lo_a(0), units(0), self(same), whole(same || TS_STAGE / (wa + wb) >= 4) {
+    sa = whole ? wa : TcKind<KIND>::NPL * pa;
+    lo_a = whole ? 2 * pa : pa;
+    const int u = TS_STAGE / (wb + (self ? 0 : sa));
+    units = u > TS_UMAX ? TS_UMAX : u / 2 * 2;
+  }
+};
+static_assert(TcShape<TC_TF32>(128, 128, false).units >= 4 && TcShape<TC_BF16X3>(128, 128, false).units >= 4,
+              "four units fit a stage");
 
 template <int KIND>
 __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
@@ -191,7 +209,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
     issued_s = 0;
     mma_steps_s = 0;
   }
-  for (int i = tid; i < 2048 / 16; i += TS_THREADS)
+  for (int i = tid; i < TS_NZERO / 16; i += TS_THREADS)
     reinterpret_cast<uint4*>(smem + TS_ZERO)[i] = make_uint4(0, 0, 0, 0);
   fence_async_smem();   // the zeros are read by the tensor cores
   if (warp == 1) {
@@ -239,8 +257,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
       const TcItem it = items[ii];
       const TcPair pr = prs[it.pair];
       const TcFrag A = fr[pr.a], B = fr[pr.b];
-      const int ua = A.rows * UB * NPL, ub = B.rows * UB * NPL;   // bytes of a unit
-      const int U = tc_units<KIND>(A.rows, B.rows);
+      const TcShape<KIND> sh(A.rows, B.rows, pr.a == pr.b);
+      const int U = sh.units;
       const int nu = (it.r1 - it.r0) * it.m;
       for (int k0 = 0; k0 < nu; k0 += U, ++g) {
         const int s = g % TS_NSTAGE, u = g / TS_NSTAGE;
@@ -252,7 +270,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
         }
         const int nk = min(U, nu - k0);
         const uint32_t mb = smem_u32(&full[s]);
-        if (lane == 0) mbar_arrive_expect(mb, (uint32_t)(nk * (ua + 2 * ub)));
+        if (lane == 0) mbar_arrive_expect(mb, (uint32_t)(nk * (sh.wb + (sh.self ? 0 : sh.sa))));
         __syncwarp();
         const int row0 = k0 / it.m, x0 = k0 - row0 * it.m;
         const int nruns = (k0 + nk - 1) / it.m - row0 + 1;   // <= U <= 32
@@ -264,14 +282,19 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
           const int y = r % it.leny, z = r / it.leny;
           const long long qa = ((long long)(it.la[2] + z) * A.dext1 + it.la[1] + y) * A.nux + it.la[0] + x;
           const long long qb = ((long long)(it.lb[2] + z) * B.dext1 + it.lb[1] + y) * B.nux + it.lb[0] + x;
-          const unsigned char* sa = planes + A.base / KT::SHARE + qa * ua;
-          const unsigned char* sb = planes + B.base / KT::SHARE + qb * ub;
-          const uint32_t d = smem_u32(smem + (size_t)s * TS_STAGE);
-          const uint32_t dB = d + (uint32_t)(U * ua), dH = dB + (uint32_t)(U * ub);
-          const uint32_t oa = (uint32_t)((ks - k0) * ua), ob = (uint32_t)((ks - k0) * ub);
-          bulk_g2s(d + oa, sa, (uint32_t)(run * ua), mb);
-          bulk_g2s(dB + ob, sb, (uint32_t)(run * ub), mb);
-          bulk_g2s(dH + ob, sb + 2 / KT::SHARE * B.npl2, (uint32_t)(run * ub), mb);
+          const unsigned char* sa = planes + A.base / KT::SHARE + qa * sh.wa;
+          const unsigned char* sb = planes + B.base / KT::SHARE + qb * sh.wb;
+          const uint32_t dB = smem_u32(smem + (size_t)s * TS_STAGE), dA = dB + (uint32_t)(U * sh.wb);
+          bulk_g2s(dB + (uint32_t)((ks - k0) * sh.wb), sb, (uint32_t)(run * sh.wb), mb);
+          const uint32_t oa = dA + (uint32_t)((ks - k0) * sh.sa);
+          if (sh.whole && !sh.self) {
+            bulk_g2s(oa, sa, (uint32_t)(run * sh.wa), mb);
+          } else if (!sh.self) {
+            for (int k = 0; k < run; ++k)
+#pragma unroll
+              for (int pl = 0; pl < NPL; ++pl)
+                bulk_g2s(oa + (uint32_t)(k * sh.sa + pl * sh.pa), sa + k * sh.wa + pl * 2 * sh.pa, (uint32_t)sh.pa, mb);
+          }
         }
         if (lane == 0) *(volatile int*)&issued_s = g + 1;
       }
@@ -291,23 +314,23 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
         const TcItem it = items[ii];
         const TcPair pr = prs[it.pair];
         const int ra = fr[pr.a].rows, rb = fr[pr.b].rows;
-        const int ua = ra * UB * NPL, ub = rb * UB * NPL, U = tc_units<KIND>(ra, rb);
+        const TcShape<KIND> sh(ra, rb, pr.a == pr.b);
+        const int U = sh.units;
         const int nu = (it.r1 - it.r0) * it.m;
-        const uint32_t N = (uint32_t)((rb + 15) / 16 * 16);
-        const uint32_t idesc = instr_desc(FMT, 128, N);
+        const uint32_t idesc = instr_desc(FMT, 128, (uint32_t)(2 * rb));
         const int b = item_no & 1, ubar = item_no >> 1;
         if (ubar > 0 && !(ok = wait(&acc_empty[b], (uint32_t)((ubar - 1) & 1)))) break;
         tc_fence_after();
-        const uint32_t dS = tmem + (uint32_t)(b * TS_ACC_COLS), dH = dS + N;
+        const uint32_t dst = tmem + (uint32_t)(b * TS_ACC_COLS);   // S, then H
         for (int k0 = 0; k0 < nu; k0 += U, ++g) {
           const int s = g % TS_NSTAGE, u = g / TS_NSTAGE;
           if (!(ok = wait(&full[s], (uint32_t)(u & 1)))) break;
           tc_fence_after();
           const int nk = min(U, nu - k0);
           const uint32_t zero = smem_u32(smem + TS_ZERO);
-          uint32_t a = smem_u32(smem + (size_t)s * TS_STAGE);
-          uint32_t p = a + (uint32_t)(U * ua), h = p + (uint32_t)(U * ub);
-          const uint32_t la = (uint32_t)(ra * UB), lb = (uint32_t)(rb * UB);   // hi -> lo
+          uint32_t p = smem_u32(smem + (size_t)s * TS_STAGE);
+          uint32_t a = sh.self ? p : p + (uint32_t)(U * sh.wb);
+          const uint32_t la = (uint32_t)sh.lo_a, lb = (uint32_t)(sh.wb / 2);   // hi -> lo
           for (int q = 0; q < nk; q += KU) {
             // TF32: both cores of the unit; BF16: this unit's core and the next
             // unit's (zeros after the last)
@@ -315,21 +338,16 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
             auto desc = [&](uint32_t addr, uint32_t ustep) {
               return smem_desc(addr, KU == 1 ? 128u : two ? ustep : zero - addr, SBO);
             };
-            const uint64_t a0 = desc(a, (uint32_t)ua), p0 = desc(p, (uint32_t)ub), h0 = desc(h, (uint32_t)ub);
+            const uint64_t a0 = desc(a, (uint32_t)sh.sa), p0 = desc(p, (uint32_t)sh.wb);
             const uint32_t acc = (k0 > 0 || q > 0) ? 1u : 0u;
-            mma<KIND>(dS, a0, p0, idesc, acc);
-            mma<KIND>(dH, a0, h0, idesc, acc);
+            mma<KIND>(dst, a0, p0, idesc, acc);
             if constexpr (NPL == 2) {
-              const uint64_t a1 = desc(a + la, (uint32_t)ua), p1 = desc(p + lb, (uint32_t)ub),
-                             h1 = desc(h + lb, (uint32_t)ub);
-              mma<KIND>(dS, a0, p1, idesc, 1u);
-              mma<KIND>(dH, a0, h1, idesc, 1u);
-              mma<KIND>(dS, a1, p0, idesc, 1u);
-              mma<KIND>(dH, a1, h0, idesc, 1u);
+              const uint64_t a1 = desc(a + la, (uint32_t)sh.sa), p1 = desc(p + lb, (uint32_t)sh.wb);
+              mma<KIND>(dst, a0, p1, idesc, 1u);
+              mma<KIND>(dst, a1, p0, idesc, 1u);
             }
-            a += (uint32_t)(KU * ua);
-            p += (uint32_t)(KU * ub);
-            h += (uint32_t)(KU * ub);
+            a += (uint32_t)(KU * sh.sa);
+            p += (uint32_t)(KU * sh.wb);
           }
           mma_commit(smem_u32(&empty[s]));
           *(volatile int*)&mma_steps_s = g + 1;
@@ -352,7 +370,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1) tc_contract_kernel(
       if (ii < 0) break;
       const TcItem it = items[ii];
       const TcPair pr = prs[it.pair];
-      const int na = fr[pr.a].n, nb = fr[pr.b].n, N = (fr[pr.b].rows + 15) / 16 * 16;
+      const int na = fr[pr.a].n, nb = fr[pr.b].n, N = fr[pr.b].rows;
       const int b = item_no & 1, ubar = item_no >> 1;
       ok = __all_sync(0xffffffffu, wait(&acc_full[b], (uint32_t)(ubar & 1)));
       if (!ok) break;
@@ -587,7 +605,6 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
     u.tile0 = tiles;
     u.base = t->plane_bytes;
     q.base = u.base;
-    q.npl2 = (long long)u.ntiles * 128 * q.rows;
     tiles += u.ntiles;
     t->plane_bytes += (long long)u.ntiles * 64 * q.rows * 8;
     t->frags.push_back(q);
