@@ -10,7 +10,7 @@
 // layout (core matrices of 8 states x 16 bytes; TF32 two cores per 8-state
 // group, BF16 one), the rows of phi and of H phi one after the other (BF16 hi+lo:
 // both hi, then both lo): one operand of 2 rows_pad MMA columns, since an MMA of 128
-// rows takes the same 33 ns for any number of them.  Both fragments of a pair share
+// rows takes about the same 33 ns for any number of them.  Both fragments of a pair share
 // the grid's units and are zero outside their own boxes, so the pair sums over the
 // units that both touch, and a run of units along the axis is one bulk copy: no
 // conversion stands between the copies and the MMAs.  Of a only phi is wanted: its
@@ -18,7 +18,7 @@
 // a unit), where they are small; a pair of a fragment with itself takes a's rows
 // from b's copy.  56 uneven boxes with 826 pairs: contraction 2.13 ms in TF32 and 1.69
 // in BF16 hi+lo with a conversion of FP32 rows in shared memory for every pair, 0.58
-// and 0.74 ms with phi and H phi as separate planes and MMAs, 0.53 and 0.56 ms now.
+// and 0.74 ms with phi and H phi as separate planes and MMAs, 0.51 and 0.54 ms now.
 //
 // A persistent CTA per SM takes items (pair, rows of units of a piece) from a
 // global counter, the largest first, through a warp-specialised pipeline: a
@@ -561,10 +561,9 @@ ofm_status ofm_plan_extra(ofm_ctx* c) {
   // planes come to the fewest bytes (x among equals).  A box of 18 points at an odd
   // offset touches four units, 32 points; along an axis that it spans whole, or
   // shares whole with its neighbours, hardly any point is padding.  Chains along
-  // x in BF16 hi+lo, units always along x and now: 31 boxes of 16 x 32 x 32, 32
-  // states, 308 and 201 us; 64 of 16 x 20 x 32, 16 states, 326 and 216 us; 4 of
-  // 16 x 12 x 12, 6 states, 69 and 55 us (with the unit's hi and lo rows together,
-  // one copy instead of two).
+  // x in BF16 hi+lo, units always along x and along the axis taken: 31 boxes of 16 x
+  // 32 x 32, 32 states, 314 and 201 us; 64 of 16 x 20 x 32, 16 states, 328 and 216 us;
+  // 4 of 16 x 12 x 12, 6 states, 67 and 58 us.
   const int* gn = c->grid.n;
   const UnitAxis uax[3] = {UnitAxis(c->frags, gn[0], 0), UnitAxis(c->frags, gn[1], 1), UnitAxis(c->frags, gn[2], 2)};
   double cost_of[3] = {0, 0, 0};
